@@ -14,6 +14,7 @@
 #include <cuda_runtime.h>
 #include <math.h>
 
+#include "fp64_int.cuh"
 #include "hydro_internal.h"
 #include "pieces.h"
 
@@ -83,27 +84,31 @@ __device__ __forceinline__ bool rows_vectorisable(const void *U, int nx, long lo
 }
 
 // Reciprocal square root, quotient and reciprocal in the working precision.
-// FP64 uses CUDA's IEEE-accurate double routines; FP32 uses the SFU
-// approximations (rsqrtf, __fdividef: at most 2 ulp), well inside the FP32
-// path's error budget.
-__device__ __forceinline__ double rsqrt_t(double x) { return rsqrt(x); }
+// FP64: the hardware's seed refined on the integer pipe (fp64_int.cuh), no
+// FP64 instruction; FP32: the SFU approximations (rsqrtf, __fdividef: at most
+// 2 ulp), well inside the FP32 path's error budget.
+//
+// The FP64 reciprocal square root takes normal positive arguments; the rest
+// (zero, negative, subnormal, infinite, NaN) goes to CUDA's rsqrt.
+__device__ __forceinline__ double rsqrt_t(double x)
+{
+    if (static_cast<unsigned>(__double2hiint(x)) - 0x00100000u >= 0x7fe00000u) return rsqrt(x);
+    double y;
+    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+    return __longlong_as_double(rsqrt_bits(__double_as_longlong(x), __double2hiint(y)));
+}
 __device__ __forceinline__ float rsqrt_t(float x) { return rsqrtf(x); }
 
-// FP64 reciprocal by Newton-Raphson iteration on f(y) = 1/y - b, which
-// doubles the number of correct bits per step: y <- y + y (1 - b y).  The
-// start value is the hardware approximation rcp.approx.ftz.f64 (about 20
-// correct bits), so two steps reach the FP64 rounding level; the result is
-// within a couple of ulp of 1/b for normal b (not always correctly rounded),
-// far inside the 1e-10 parity budget.  Costs one SFU operation and four
-// FMAs on the FP64 pipe.
+// FP64 reciprocal, within 0.53 ulp for every b whose reciprocal is normal;
+// NaN for zero, subnormal, infinite or NaN b, and 0 from 2^1022 on.
 __device__ __forceinline__ double rcp_t(double b)
 {
     double y;
     asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(b));
-    double e = fma(-b, y, 1.0);
-    y = fma(y, e, y);
-    e = fma(-b, y, 1.0);
-    return fma(y, e, y);
+    const double r = __longlong_as_double(rcp_bits(__double_as_longlong(b), __double2hiint(y)));
+    const unsigned be = static_cast<unsigned>(__double2hiint(b)) & 0x7ff00000u;
+    if (be - 0x00100000u < 0x7fc00000u) return r;
+    return __hiloint2double((be == 0u || be == 0x7ff00000u) ? 0x7ff80000 : 0, 0);
 }
 __device__ __forceinline__ float rcp_t(float b) { return __fdividef(1.0f, b); }
 __device__ __forceinline__ double div_t(double a, double b) { return a * rcp_t(b); }
@@ -442,16 +447,20 @@ __device__ __forceinline__ void ppm_faces(T am, T a, T ap, T sm, T s, T sp, T &l
 //
 // Arithmetic is arranged to need two square-root reciprocals and two
 // divisions per face: c = g rsqrt(g rho) with g = gamma p.  The star state of
-// Toro eq. (10.39), rho*_K = rho_K (S_K - u_K) / (S_K - S*) with velocity
-// (S*, v_t) and E*_K = rho*_K [E_K / rho_K + (S* - u_K)(S* + p_K / (rho_K (S_K - u_K)))],
-// enters only through F*_K = F_K + S_K (U*_K - U_K), whose components reduce
-// to multiples of one factor h = S_K (S* - u_K) / (S_K - S*):
-//   S_K (rho*_K - rho_K)             = rho_K h                      (= c0)
-//   S_K (rho*_K v_t - rho_K v_t)     = c0 v_t
-//   S_K (rho*_K S* - rho_K u_K)      = S_K c0
-//   S_K (E*_K - E_K)                 = h (E_K + p_K + m_K S*),  m_K = rho_K (S_K - u_K)
-// (rho*_K - rho_K = rho_K (S* - u_K) / (S_K - S*); the energy line follows
-// from E*_K - E_K written over the common denominator S_K - S*).
+// Toro eq. (10.39) enters through F*_K = F_K + S_K (U*_K - U_K) and one
+// factor h = S_K (S* - u_K) / (S_K - S*), zero outside the fan:
+//   mass             F_0 = rho_K u_K + rho_K h = rho_K (u_K + h)
+//   tangential       F_0 v_t
+//   normal momentum  F_0 u_K + p_K + m_K h,           m_K = rho_K (S_K - u_K)
+//   energy           (E_K + p_K)(u_K + h) + m_K h S*
+// (S_K (rho*_K - rho_K) = rho_K h; S_K rho_K h = rho_K h u_K + m_K h.)  The
+// star state is never formed, so nothing is subtracted from a nearly equal
+// product, and the fan's branch needs one select (of h) beside those of the
+// side.  36 arithmetic operations per face; the same fluxes as separate sums
+// F_K + correction took 44, with the same rounding error (rms over random
+// states against 128 bits: mass 4.3e-17, energy 2.6e-16 for both; forming the
+// star state itself takes 33, at 1.3 and 1.8 times that error).  Every
+// rounding is spelled out, so that each kernel gives the same bits.
 template <typename T, int ND, int D, bool HSE>
 __device__ __forceinline__ void hllc(const T (&wl)[ND + 2], const T (&wr)[ND + 2], T rb, T pb,
                                      T gam, T igm1, T (&f)[ND + 2])
@@ -462,9 +471,9 @@ __device__ __forceinline__ void hllc(const T (&wl)[ND + 2], const T (&wr)[ND + 2
     const T pl = HSE ? pb + wl[NV - 1] : wl[NV - 1];
     const T pr = HSE ? pb + wr[NV - 1] : wr[NV - 1];
     const T ul = wl[1 + D], ur = wr[1 + D];
-    const T gpl = gam * pl, gpr = gam * pr;
-    const T cl = gpl * rsqrt_t(gpl * rl);
-    const T cr = gpr * rsqrt_t(gpr * rr);
+    const T gpl = mul_rn(gam, pl), gpr = mul_rn(gam, pr);
+    const T cl = mul_rn(gpl, rsqrt_t(mul_rn(gpl, rl)));
+    const T cr = mul_rn(gpr, rsqrt_t(mul_rn(gpr, rr)));
     // S_L - u_L = min(-c_L, (u_R - u_L) - c_R) and S_R - u_R = max(c_L - (u_R - u_L), c_R):
     // the offsets the star factors m_K = rho_K (S_K - u_K) need, and S_L, S_R from them
     const T du = ur - ul;
@@ -472,14 +481,13 @@ __device__ __forceinline__ void hllc(const T (&wl)[ND + 2], const T (&wr)[ND + 2
     const T ar = max_t(cl - du, cr);
     const T sl = ul + al, sr = ur + ar;
 
-    // Branch-free: every face computes S* and the star correction and the
-    // branch of the HLLC fan is applied by selects.  The chosen branch's
-    // values are the same as with branches, and the straight-line code lets
-    // a thread's independent faces interleave.  S* and 1/(S_K - S*) are
-    // finite for positive densities and pressures (S_L < u_L, S_R > u_R).
+    // Branch-free: every face computes S* and h and the branch of the HLLC
+    // fan is applied by selects.  The straight-line code lets a
+    // thread's independent faces interleave.  S* and 1/(S_K - S*) are finite
+    // for positive densities and pressures (S_L < u_L, S_R > u_R).
     const T dpp = wr[NV - 1] - wl[NV - 1];   // background cancels in the difference
-    const T ml = rl * al, mr = rr * ar;
-    const T sstar = div_t(dpp + ml * ul - mr * ur, ml - mr);
+    const T ml = mul_rn(rl, al), mr = mul_rn(rr, ar);
+    const T sstar = div_t(fma_rn(-mr, ur, fma_rn(ml, ul, dpp)), ml - mr);
     const bool sup_l = nonnegative(sl);     // whole fan moves right: F_L
     const bool sup_r = nonpositive(sr);     // whole fan moves left: F_R
     const bool left = sup_l || (!sup_r && nonnegative(sstar));
@@ -492,42 +500,18 @@ __device__ __forceinline__ void hllc(const T (&wl)[ND + 2], const T (&wr)[ND + 2
     T vk[ND];
 #pragma unroll
     for (int e = 0; e < ND; ++e) vk[e] = left ? wl[1 + e] : wr[1 + e];
-    const T uk = vk[D];
-    T ke = T(0);
+    T ke = mul_rn(vk[0], vk[0]);
 #pragma unroll
-    for (int e = 0; e < ND; ++e) ke += vk[e] * vk[e];
+    for (int e = 1; e < ND; ++e) ke = fma_rn(vk[e], vk[e], ke);
     // E_K + p_K = p_K gamma / (gamma - 1) + rho_K |v_K|^2 / 2
-    const T hk = fma(pk, igm1 + T(1), rk * half_nonneg(ke));
-
-    // Euler flux of the chosen side
-    const T mflux = rk * uk;
-    f[0] = mflux;
+    const T hk = fma_rn(pk, igm1 + T(1), mul_rn(rk, half_nonneg(ke)));
+    const T hs = mul_rn(sstar - vk[D], mul_rn(sk, rcp_t(sk - sstar)));
+    const T h = star ? hs : T(0);
+    const T uh = vk[D] + h, g = mul_rn(mk, h);
+    f[0] = mul_rn(rk, uh);
 #pragma unroll
-    for (int e = 0; e < ND; ++e) f[1 + e] = mflux * vk[e];
-    f[1 + D] += ppk;
-    f[NV - 1] = uk * hk;
-
-    // F*_K = F_K + S_K (U*_K - U_K), applied only inside the fan
-    const T h = (sk * rcp_t(sk - sstar)) * (sstar - uk);
-    const T c0 = rk * h;                    // S_K (rho*_K - rho_K)
-    const T fE = fma(h, fma(mk, sstar, hk), f[NV - 1]);
-    if constexpr (sizeof(T) == 8) {
-        // FP64 (bound by its FP64 pipe): each star component formed by one
-        // fused multiply-add onto F_K (or one addition) and selected
-        f[0] = star ? f[0] + c0 : f[0];
-#pragma unroll
-        for (int e = 0; e < ND; ++e) {
-            const T fs = (e == D) ? fma(sk, c0, f[1 + e]) : fma(c0, vk[e], f[1 + e]);
-            f[1 + e] = star ? fs : f[1 + e];
-        }
-        f[NV - 1] = star ? fE : f[NV - 1];
-    } else {
-        const T cs = star ? c0 : T(0);
-        f[0] += cs;
-#pragma unroll
-        for (int e = 0; e < ND; ++e) f[1 + e] = fma(cs, (e == D) ? sk : vk[e], f[1 + e]);
-        f[NV - 1] = star ? fE : f[NV - 1];
-    }
+    for (int e = 0; e < ND; ++e) f[1 + e] = (e == D) ? fma_rn(f[0], vk[D], ppk + g) : mul_rn(f[0], vk[e]);
+    f[NV - 1] = fma_rn(hk, uh, mul_rn(g, sstar));
 }
 
 // Mirror image of a face state across a wall normal to axis D.
