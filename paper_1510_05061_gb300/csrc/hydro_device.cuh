@@ -456,62 +456,139 @@ __device__ __forceinline__ void ppm_faces(T am, T a, T ap, T sm, T s, T sp, T &l
 // (S_K (rho*_K - rho_K) = rho_K h; S_K rho_K h = rho_K h u_K + m_K h.)  The
 // star state is never formed, so nothing is subtracted from a nearly equal
 // product, and the fan's branch needs one select (of h) beside those of the
-// side.  36 arithmetic operations per face; the same fluxes as separate sums
-// F_K + correction took 44, with the same rounding error (rms over random
-// states against 128 bits: mass 4.3e-17, energy 2.6e-16 for both; forming the
-// star state itself takes 33, at 1.3 and 1.8 times that error).  Every
-// rounding is spelled out, so that each kernel gives the same bits.
-template <typename T, int ND, int D, bool HSE>
-__device__ __forceinline__ void hllc(const T (&wl)[ND + 2], const T (&wr)[ND + 2], T rb, T pb,
-                                     T gam, T igm1, T (&f)[ND + 2])
+// side.  36 instructions on the FP64 pipe per face; the same fluxes as
+// separate sums F_K + correction took 44, with the same rounding error (rms
+// over random states against 128 bits: mass 4.3e-17, energy 2.6e-16 for both;
+// forming the star state itself takes 33, at 1.3 and 1.8 times that error).
+// Every rounding is spelled out, so that each kernel gives the same bits.
+template <int ND, int D, bool HSE>
+__device__ __forceinline__ void hllc_f64(const double (&wl)[ND + 2], const double (&wr)[ND + 2], double rb, double pb,
+                                         double gam, double igm1, double (&f)[ND + 2])
 {
     constexpr int NV = ND + 2;
-    const T rl = HSE ? rb + wl[0] : wl[0];
-    const T rr = HSE ? rb + wr[0] : wr[0];
-    const T pl = HSE ? pb + wl[NV - 1] : wl[NV - 1];
-    const T pr = HSE ? pb + wr[NV - 1] : wr[NV - 1];
-    const T ul = wl[1 + D], ur = wr[1 + D];
-    const T gpl = mul_rn(gam, pl), gpr = mul_rn(gam, pr);
-    const T cl = mul_rn(gpl, rsqrt_t(mul_rn(gpl, rl)));
-    const T cr = mul_rn(gpr, rsqrt_t(mul_rn(gpr, rr)));
+    const double rl = HSE ? rb + wl[0] : wl[0];
+    const double rr = HSE ? rb + wr[0] : wr[0];
+    const double pl = HSE ? pb + wl[NV - 1] : wl[NV - 1];
+    const double pr = HSE ? pb + wr[NV - 1] : wr[NV - 1];
+    const double ul = wl[1 + D], ur = wr[1 + D];
+    const double gpl = mul_rn(gam, pl), gpr = mul_rn(gam, pr);
+    const double cl = mul_rn(gpl, rsqrt_t(mul_rn(gpl, rl)));
+    const double cr = mul_rn(gpr, rsqrt_t(mul_rn(gpr, rr)));
     // S_L - u_L = min(-c_L, (u_R - u_L) - c_R) and S_R - u_R = max(c_L - (u_R - u_L), c_R):
     // the offsets the star factors m_K = rho_K (S_K - u_K) need, and S_L, S_R from them
-    const T du = ur - ul;
-    const T al = min_t(-cl, du - cr);
-    const T ar = max_t(cl - du, cr);
-    const T sl = ul + al, sr = ur + ar;
+    const double du = ur - ul;
+    const double al = min_t(-cl, du - cr);
+    const double ar = max_t(cl - du, cr);
+    const double sl = ul + al, sr = ur + ar;
 
     // Branch-free: every face computes S* and h and the branch of the HLLC
     // fan is applied by selects.  The straight-line code lets a
     // thread's independent faces interleave.  S* and 1/(S_K - S*) are finite
     // for positive densities and pressures (S_L < u_L, S_R > u_R).
-    const T dpp = wr[NV - 1] - wl[NV - 1];   // background cancels in the difference
-    const T ml = mul_rn(rl, al), mr = mul_rn(rr, ar);
-    const T sstar = div_t(fma_rn(-mr, ur, fma_rn(ml, ul, dpp)), ml - mr);
+    const double dpp = wr[NV - 1] - wl[NV - 1];   // background cancels in the difference
+    const double ml = mul_rn(rl, al), mr = mul_rn(rr, ar);
+    const double sstar = div_t(fma_rn(-mr, ur, fma_rn(ml, ul, dpp)), ml - mr);
     const bool sup_l = nonnegative(sl);     // whole fan moves right: F_L
     const bool sup_r = nonpositive(sr);     // whole fan moves left: F_R
     const bool left = sup_l || (!sup_r && nonnegative(sstar));
     const bool star = !sup_l && !sup_r;
-    const T rk = left ? rl : rr;
-    const T pk = left ? pl : pr;
-    const T ppk = left ? wl[NV - 1] : wr[NV - 1];
-    const T sk = left ? sl : sr;
-    const T mk = left ? ml : mr;
-    T vk[ND];
+    const double rk = left ? rl : rr;
+    const double pk = left ? pl : pr;
+    const double ppk = left ? wl[NV - 1] : wr[NV - 1];
+    const double sk = left ? sl : sr;
+    const double mk = left ? ml : mr;
+    double vk[ND];
 #pragma unroll
     for (int e = 0; e < ND; ++e) vk[e] = left ? wl[1 + e] : wr[1 + e];
-    T ke = mul_rn(vk[0], vk[0]);
+    double ke = mul_rn(vk[0], vk[0]);
 #pragma unroll
     for (int e = 1; e < ND; ++e) ke = fma_rn(vk[e], vk[e], ke);
     // E_K + p_K = p_K gamma / (gamma - 1) + rho_K |v_K|^2 / 2
-    const T hk = fma_rn(pk, igm1 + T(1), mul_rn(rk, half_nonneg(ke)));
-    const T hs = mul_rn(sstar - vk[D], mul_rn(sk, rcp_t(sk - sstar)));
-    const T h = star ? hs : T(0);
-    const T uh = vk[D] + h, g = mul_rn(mk, h);
+    const double hk = fma_rn(pk, igm1 + 1.0, mul_rn(rk, half_nonneg(ke)));
+    const double hs = mul_rn(sstar - vk[D], mul_rn(sk, rcp_t(sk - sstar)));
+    const double h = star ? hs : 0.0;
+    const double uh = vk[D] + h, g = mul_rn(mk, h);
     f[0] = mul_rn(rk, uh);
 #pragma unroll
     for (int e = 0; e < ND; ++e) f[1 + e] = (e == D) ? fma_rn(f[0], vk[D], ppk + g) : mul_rn(f[0], vk[e]);
     f[NV - 1] = fma_rn(hk, uh, mul_rn(g, sstar));
+}
+
+// The FP32 flux: F_K plus the correction S_K (U*_K - U_K) in multiples of the
+// same h, the components' increments added one by one.  (The FP64 grouping
+// saves nothing here: 0 to 1 % of the step, with other bits.)
+template <int ND, int D, bool HSE>
+__device__ __forceinline__ void hllc_f32(const float (&wl)[ND + 2], const float (&wr)[ND + 2], float rb, float pb,
+                                         float gam, float igm1, float (&f)[ND + 2])
+{
+    constexpr int NV = ND + 2;
+    const float rl = HSE ? rb + wl[0] : wl[0];
+    const float rr = HSE ? rb + wr[0] : wr[0];
+    const float pl = HSE ? pb + wl[NV - 1] : wl[NV - 1];
+    const float pr = HSE ? pb + wr[NV - 1] : wr[NV - 1];
+    const float ul = wl[1 + D], ur = wr[1 + D];
+    const float gpl = gam * pl, gpr = gam * pr;
+    const float cl = gpl * rsqrt_t(gpl * rl);
+    const float cr = gpr * rsqrt_t(gpr * rr);
+    // S_L - u_L = min(-c_L, (u_R - u_L) - c_R) and S_R - u_R = max(c_L - (u_R - u_L), c_R):
+    // the offsets the star factors m_K = rho_K (S_K - u_K) need, and S_L, S_R from them
+    const float du = ur - ul;
+    const float al = min_t(-cl, du - cr);
+    const float ar = max_t(cl - du, cr);
+    const float sl = ul + al, sr = ur + ar;
+
+    // Branch-free: every face computes S* and the star correction and the
+    // branch of the HLLC fan is applied by selects.  The chosen branch's
+    // values are the same as with branches, and the straight-line code lets
+    // a thread's independent faces interleave.  S* and 1/(S_K - S*) are
+    // finite for positive densities and pressures (S_L < u_L, S_R > u_R).
+    const float dpp = wr[NV - 1] - wl[NV - 1];   // background cancels in the difference
+    const float ml = rl * al, mr = rr * ar;
+    const float sstar = div_t(dpp + ml * ul - mr * ur, ml - mr);
+    const bool sup_l = nonnegative(sl);     // whole fan moves right: F_L
+    const bool sup_r = nonpositive(sr);     // whole fan moves left: F_R
+    const bool left = sup_l || (!sup_r && nonnegative(sstar));
+    const bool star = !sup_l && !sup_r;
+    const float rk = left ? rl : rr;
+    const float pk = left ? pl : pr;
+    const float ppk = left ? wl[NV - 1] : wr[NV - 1];
+    const float sk = left ? sl : sr;
+    const float mk = left ? ml : mr;
+    float vk[ND];
+#pragma unroll
+    for (int e = 0; e < ND; ++e) vk[e] = left ? wl[1 + e] : wr[1 + e];
+    const float uk = vk[D];
+    float ke = 0.0f;
+#pragma unroll
+    for (int e = 0; e < ND; ++e) ke += vk[e] * vk[e];
+    // E_K + p_K = p_K gamma / (gamma - 1) + rho_K |v_K|^2 / 2
+    const float hk = fma(pk, igm1 + 1.0f, rk * half_nonneg(ke));
+
+    // Euler flux of the chosen side
+    const float mflux = rk * uk;
+    f[0] = mflux;
+#pragma unroll
+    for (int e = 0; e < ND; ++e) f[1 + e] = mflux * vk[e];
+    f[1 + D] += ppk;
+    f[NV - 1] = uk * hk;
+
+    // F*_K = F_K + S_K (U*_K - U_K), applied only inside the fan
+    const float h = (sk * rcp_t(sk - sstar)) * (sstar - uk);
+    const float c0 = rk * h;                    // S_K (rho*_K - rho_K)
+    const float fE = fma(h, fma(mk, sstar, hk), f[NV - 1]);
+    const float cs = star ? c0 : 0.0f;
+    f[0] += cs;
+#pragma unroll
+    for (int e = 0; e < ND; ++e) f[1 + e] = fma(cs, (e == D) ? sk : vk[e], f[1 + e]);
+    f[NV - 1] = star ? fE : f[NV - 1];
+}
+
+template <typename T, int ND, int D, bool HSE>
+__device__ __forceinline__ void hllc(const T (&wl)[ND + 2], const T (&wr)[ND + 2], T rb, T pb, T gam, T igm1,
+                                     T (&f)[ND + 2])
+{
+    if constexpr (sizeof(T) == 8) hllc_f64<ND, D, HSE>(wl, wr, rb, pb, gam, igm1, f);
+    else hllc_f32<ND, D, HSE>(wl, wr, rb, pb, gam, igm1, f);
 }
 
 // Mirror image of a face state across a wall normal to axis D.
