@@ -183,7 +183,8 @@ int hydro_get_fields(hydro_sim *sim, int what, double *host_dst);
    from the host. */
 int hydro_debug_poke(hydro_sim *sim, int var, long cell, double v);
 
-/* Select the 3D z-chunk length (planes per CTA); 0 restores the default.
+/* Select the 3D z-chunk length (planes per CTA); 0 restores the default
+   (the balanced grid; z-chunks for the paired-cell variants).
    A negative value selects the balanced grid instead: as many CTAs as the
    device holds resident at once, the (tile, z-chunk) pieces taken in whole
    waves of neighbouring tiles at the same heights while at least one wave
@@ -201,8 +202,8 @@ int hydro_set_zchunk(hydro_sim *sim, int zchunk);
    hydro_batch_variant_shape.  Variants 0..3 load each staged plane
    synchronously, 4..7 (the same shapes) copy the next plane asynchronously
    one plane ahead (MUSCL-Hancock step; the other integrators use the shape
-   only).  Default: variant 7 (32 x 16) for FP32, 6 (16 x 16) for FP64, the
-   autotuner's usual choices on GB300.  Variants 3
+   only).  Default: chosen from the grid's size and the precision (FP64 mostly
+   variant 6, 16 x 16; FP32 mostly 0, 32 x 8).  Variants 3
    and 7 (32 x 16) are FP32 only.  Results do not depend on the choice
    among 0..7; the paired-cell FP32 variants 8..10 are described below. */
 int hydro_set_tile(hydro_sim *sim, int variant);

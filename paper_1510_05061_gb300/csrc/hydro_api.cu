@@ -19,6 +19,7 @@
 #include "launchers.h"
 #include "per_device.h"
 #include "pieces.h"
+#include "plan.h"
 
 using namespace hydro;
 
@@ -205,6 +206,7 @@ AuxArgs aux_args(const hydro_sim *s, void *U)
     return a;
 }
 
+// z-chunk of the kernels without a balanced grid (the paired-cell tiles)
 int default_zchunk(const hydro_sim *s)
 {
     if (s->prob.ndim == 2) return 1;
@@ -216,6 +218,17 @@ int default_zchunk(const hydro_sim *s)
     nch = std::max(nch, (long long)((nz + 63) / 64));
     nch = std::min(nch, std::max(1ll, (long long)(nz / 8)));
     return (int)((nz + nch - 1) / nch);
+}
+
+// The default z partition: the plan's, where the kernel has it.
+void set_default_partition(hydro_sim *s)
+{
+    s->balanced = 0;
+    s->zchunk = default_zchunk(s);
+    if (s->prob.scheme == HYDRO_SCHEME_CTU || pair_variant(s->variant)) return;
+    const int z = default_plan(s->prob).zchunk;
+    if (z > 0) s->zchunk = z;
+    else s->balanced = z;
 }
 
 StepArgs step_args(const hydro_sim *s, double t_end)
@@ -396,13 +409,13 @@ int init_impl(const hydro_problem *prob, void *Ua, void *Ub, void *work, const d
         s->tiles_x = tiles_along(prob->n[0], STEP2D_TX);
         s->tiles_y = tiles_along(prob->n[1], STEP2D_TY);
     } else {
-        // the autotuner's usual choice on GB300: asynchronous staging with
-        // 32 x 16 tiles (FP32) or 16 x 16 tiles (FP64)
-        s->variant = prob->precision == HYDRO_FP32 ? 7 : 6;
+        const LaunchPlan plan = default_plan(*prob);
+        s->variant = plan.variant;
         s->tiles_x = tiles_along(prob->n[0], TILE3D_SHAPES[s->variant].tx);
         s->tiles_y = tiles_along(prob->n[1], TILE3D_SHAPES[s->variant].ty);
     }
-    s->zchunk = default_zchunk(s);
+    if (prob->ndim == 2) s->zchunk = 1;
+    else set_default_partition(s);
 
     cudaError_t e = cudaMemsetAsync(s->work, 0, s->lay.total, s->stream);
     if (e != cudaSuccess) { delete s; return HYDRO_ERR_CUDA; }
@@ -630,7 +643,11 @@ int hydro_set_zchunk(hydro_sim *s, int zchunk)
         return HYDRO_OK;
     }
     if (s->prob.ndim == 2) return zchunk <= 1 ? HYDRO_OK : HYDRO_ERR_INVALID_ARG;
-    s->zchunk = zchunk == 0 ? default_zchunk(s) : std::min(zchunk, s->prob.n[2]);
+    if (zchunk == 0) {
+        set_default_partition(s);
+        return HYDRO_OK;
+    }
+    s->zchunk = std::min(zchunk, s->prob.n[2]);
     s->balanced = 0;
     return HYDRO_OK;
 }
