@@ -19,6 +19,7 @@
 #include <vector>
 
 #include "../../include/hydro.h"
+#include "host_pages.h"
 #include "hydro_internal.h"
 #include "launchers.h"
 
@@ -753,6 +754,7 @@ int hydro_batch_get_fields(hydro_batch *b, int id, int what, double *host_dst)
         const long long m = std::min(cap, I.N - c0);
         b->launches += 1;
         cudaError_t e = launch_fields(a, stg, c0, m, what, b->stream);
+        if (c0 == 0) touch_pages(host_dst, sizeof(double) * (size_t)I.nvar * I.N);   // beside the kernel
         for (int q = 0; q < I.nvar && e == cudaSuccess; ++q)
             e = cudaMemcpyAsync(host_dst + (size_t)q * I.N + c0, stg + (size_t)q * m, sizeof(double) * m,
                                 cudaMemcpyDeviceToHost, b->stream);
@@ -769,6 +771,7 @@ int hydro_batch_get_state(hydro_batch *b, int id, void *host_dst)
     Ctrl c;
     int rc = read_inst_ctrl(b, I, &c);
     if (rc) return rc;
+    touch_pages(host_dst, I.state_bytes);
     cudaError_t e = cudaMemcpyAsync(host_dst, I.buf[state_index(I, c.step)], I.state_bytes, cudaMemcpyDeviceToHost,
                                     b->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(b->stream);

@@ -15,6 +15,7 @@
 #include <vector>
 
 #include "../../include/hydro.h"
+#include "host_pages.h"
 #include "hydro_internal.h"
 #include "launchers.h"
 #include "per_device.h"
@@ -575,6 +576,7 @@ void *hydro_current(hydro_sim *s) { return s ? s->buf[s->cur] : nullptr; }
 int hydro_get_state(hydro_sim *s, void *host_dst)
 {
     if (!s || !host_dst) return HYDRO_ERR_INVALID_ARG;
+    touch_pages(host_dst, s->state_bytes);
     cudaError_t e = cudaMemcpyAsync(host_dst, s->buf[s->cur], s->state_bytes, cudaMemcpyDeviceToHost,
                                     s->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s->stream);
@@ -611,6 +613,7 @@ int hydro_get_fields(hydro_sim *s, int what, double *host_dst)
         const long long m = std::min(cap, s->N - c0);
         s->launches += 1;
         cudaError_t e = launch_fields(a, stg, c0, m, what, s->stream);
+        if (c0 == 0) touch_pages(host_dst, sizeof(double) * (size_t)s->nvar * s->N);   // beside the kernel
         for (int q = 0; q < s->nvar && e == cudaSuccess; ++q)
             e = cudaMemcpyAsync(host_dst + (size_t)q * s->N + c0, stg + (size_t)q * m,
                                 sizeof(double) * m, cudaMemcpyDeviceToHost, s->stream);
