@@ -9,7 +9,7 @@ namespace hydro {
 template <typename T>
 static cudaError_t launch_ctu(const StepArgs &a, dim3 grid, cudaStream_t s)
 {
-    constexpr int TX = STEP2D_TX, TY = STEP2D_TY;
+    constexpr int TX = CTU2D_TX, TY = CTU2D_TY;
     auto k = ctu2d_kernel<T, TX, TY>;
     constexpr size_t smem = Ctu2DSmem<T, TX, TY>::bytes;
     static PerDeviceOnce configured;   // the attribute is per function and device

@@ -106,7 +106,7 @@ int tiles_along(int n, int t) { return (n + t - 1) / t; }
 int step_max_ctas(const hydro_problem *p)
 {
     if (p->ndim == 2)
-        return tiles_along(p->n[0], STEP2D_TX) * tiles_along(p->n[1], STEP2D_TY);
+        return std::max(tiles_along(p->n[0], STEP2D_MIN_TX) * tiles_along(p->n[1], STEP2D_MIN_TY), MARCH2D_MAX_CTAS);
     // any tile shape, zchunk >= 1: at most nz chunks
     int m = 0;
     for (int v = 0; v < TILE3D_VARIANTS; ++v)
@@ -272,7 +272,7 @@ cudaError_t launch_kernel(hydro_sim *s, const StepArgs &a, int stage)
     if (s->prob.ndim == 2 && s->prob.scheme == HYDRO_SCHEME_CTU)
         return launch_ctu2d(a, dim3(s->tiles_x * s->tiles_y, 1), s->stream, fp32);
     if (s->prob.ndim == 2)
-        return launch_step2d(a, dim3(s->tiles_x * s->tiles_y, 1), s->stream, fp32, stage, recon);
+        return launch_step2d(a, s->stream, fp32, stage, recon);
     if (s->prob.scheme == HYDRO_SCHEME_CTU) return launch_ctu3d(a, s->stream, fp32, hse);
     const dim3 grid(s->tiles_x * s->tiles_y, (s->prob.n[2] + s->zchunk - 1) / s->zchunk);
     if (stage == STAGE_HANCOCK && pair_variant(s->variant))
@@ -407,8 +407,8 @@ int init_impl(const hydro_problem *prob, void *Ua, void *Ub, void *work, const d
         if (d < prob->ndim) s->cell_volume *= s->dx[d];
     }
     if (prob->ndim == 2) {
-        s->tiles_x = tiles_along(prob->n[0], STEP2D_TX);
-        s->tiles_y = tiles_along(prob->n[1], STEP2D_TY);
+        s->tiles_x = tiles_along(prob->n[0], CTU2D_TX);
+        s->tiles_y = tiles_along(prob->n[1], CTU2D_TY);
     } else {
         const LaunchPlan plan = default_plan(*prob);
         s->variant = plan.variant;

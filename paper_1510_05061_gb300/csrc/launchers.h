@@ -8,9 +8,14 @@
 
 namespace hydro {
 
-// 2D step tile.
-constexpr int STEP2D_TX = 32;
-constexpr int STEP2D_TY = 8;
+// 2D corner transport upwind tile.
+constexpr int CTU2D_TX = 32;
+constexpr int CTU2D_TY = 8;
+// Smallest tile of the 2D step (its largest CTA count), and the most CTAs of
+// the marched 2D step.
+constexpr int STEP2D_MIN_TX = 16;
+constexpr int STEP2D_MIN_TY = 8;
+constexpr int MARCH2D_MAX_CTAS = 1024;
 
 // Tile shapes of the 3D step (TX x TY threads, one column of cells each),
 // chosen per solve or per batch by the autotuner.  The 512-thread 32 x 16
@@ -68,9 +73,12 @@ cudaError_t launch_stage3d_f64(int stage, int v, const StepArgs &a, dim3 grid, c
                                int recon);
 cudaError_t launch_stage3d_f32(int stage, int v, const StepArgs &a, dim3 grid, cudaStream_t s, bool hse,
                                int recon);
-// stage: STAGE_HANCOCK, STAGE_RK1 or STAGE_RK2; recon as above (stages only)
-cudaError_t launch_step2d(const StepArgs &a, dim3 grid, cudaStream_t s, bool fp32, int stage = STAGE_HANCOCK,
-                          int recon = RECON_PLM);
+// 2D step: stage STAGE_HANCOCK, STAGE_RK1 or STAGE_RK2; recon as above (stages
+// only); the launch shape is plan2d's
+cudaError_t launch_step2d(const StepArgs &a, cudaStream_t s, bool fp32, int stage, int recon);
+// the same step on column strips of nt - 4 columns marched along y (FP64: nt =
+// 128; FP32: 128 or 256)
+cudaError_t launch_march2d(const StepArgs &a, int nt, cudaStream_t s, bool fp32, int stage);
 
 // corner transport upwind step (2D: same tile as the 2D step; 3D: blocks of
 // cells, ctu3d_blocks of them)

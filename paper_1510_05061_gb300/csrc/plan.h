@@ -73,4 +73,41 @@ inline LaunchPlan default_plan(const hydro_problem &p)
     return best;
 }
 
+// Launch shape of the 2D step: march = threads of a marched strip, or 0 and
+// the tile (tx x ty).
+struct Plan2D {
+    int march, tx, ty;
+};
+
+// Tiles (measured, us per MUSCL-Hancock step): FP64 16 x 16 cells (512^2 152
+// against 160 with 32 x 8; 517x331 111 against 117), 16 x 8 while those fit one
+// per SM (128^2: 26 against 33); FP32 32 x 16 (384^2 12.6 against 14.5), 16 x 16
+// for the parabolic stages (1448^2 179 against 187).  A strip (linear states)
+// is taken where its modelled time, row time x (rows per CTA + 2.2), is below
+// the tiles' time per padded cell; the row times at full residency and the
+// tiles' cell times are fitted at 512^2 to 2048^2.  The crossing lies near 700^2
+// (FP64: 266 against 293) and 1024^2 (FP32: 38.3 against 37.9).
+inline Plan2D plan2d(int nx, int ny, bool fp32, bool ppm)
+{
+    constexpr int SMS = 152;
+    const auto along = [](long long n, int t) { return (n + t - 1) / t; };
+    Plan2D best{0, fp32 && !ppm ? 32 : 16, 16};
+    if (!fp32 && along(nx, 16) * along(ny, 8) <= SMS) best.ty = 8;
+    if (ppm) return best;
+    const double cells = (double)along(nx, best.tx) * best.tx * along(ny, best.ty) * best.ty;
+    double tbest = fp32 ? 4.0 + 31.5e-6 * cells : 10.0 + 525e-6 * cells;
+    struct Strip { int nt, ctas; double row; };
+    static const Strip f64[] = {{128, 3, 22.9}};
+    static const Strip f32[] = {{128, 6, 2.5}, {256, 3, 2.5}};
+    const Strip *c = fp32 ? f32 : f64;
+    for (int i = 0; i < (fp32 ? 2 : 1); ++i) {
+        const double t = c[i].row * (along(along(nx, c[i].nt - 4) * ny, SMS * c[i].ctas) + 2.2);
+        if (t < tbest) {
+            tbest = t;
+            best.march = c[i].nt;
+        }
+    }
+    return best;
+}
+
 }  // namespace hydro
