@@ -208,25 +208,34 @@ __device__ __forceinline__ float mc_slope(float dl, float dr)
     return (dl * dr > 0.0f) ? copysignf(a, dr) : 0.0f;
 }
 
-// FP64 form: the sign test, both minima, the doubling and the halving act
-// on the IEEE bit patterns (integer pipe; for non-negative doubles integer
-// order is numeric order, and adding or removing 1 in the exponent field
-// multiplies a normal number by 2 or 1/2 exactly), leaving the differences
-// and dl + dr on the FP64 pipe.  When dl and dr share a sign both are
-// nonzero and their sum is nonzero; a |dl + dr| below 2^-1021 (no normal
-// halving) gives a zero slope.
+// FP64 form, on the IEEE bit patterns with integer instructions only (for
+// non-negative doubles integer order is numeric order; adding or removing 1
+// in the exponent field multiplies a normal number by 2 or 1/2 exactly).
+// With M >= m the magnitudes of two differences of one sign, 2 m is the
+// smallest of the three candidates once M's exponent exceeds m's by three
+// (then M + m > 5 m); below that the sum aligns by at most two bits, never
+// cancels and rounds to nearest even from two or three extra bits, so the
+// slope has the bits of the FP64 instructions (a sum below 2^-1021, without a
+// normal half, gives a zero slope).  The sum was the last FP64 instruction of
+// the slope, one for each variable and axis of every predicted cell.
 __device__ __forceinline__ double mc_slope(double dl, double dr)
 {
-    constexpr long long ABS = 0x7fffffffffffffffll, ONE_EXP = 1ll << 52;
-    const long long bl = __double_as_longlong(dl), br = __double_as_longlong(dr);
-    const long long al = bl & ABS, ar = br & ABS;
-    const bool same = ((bl ^ br) >= 0) && al != 0 && ar != 0;
-    const long long m = min(al, ar);
-    const long long twice = m < (0x7fell << 52) ? m + ONE_EXP : m;       // 2 min(|dl|, |dr|)
-    const long long as = __double_as_longlong(dl + dr) & ABS;
-    const long long half = as >= (2ll << 52) ? as - ONE_EXP : 0ll;        // |dl + dr| / 2
-    const double a = __longlong_as_double(min(twice, half));
-    return same ? copysign(a, dr) : 0.0;
+    using u64 = unsigned long long;
+    constexpr u64 ABS = 0x7fffffffffffffffull, ONE_EXP = 1ull << 52, MANT = ONE_EXP - 1;
+    const u64 bl = __double_as_longlong(dl), br = __double_as_longlong(dr);
+    const u64 al = bl & ABS, ar = br & ABS;
+    const bool same = static_cast<long long>(bl ^ br) >= 0 && al != 0 && ar != 0;
+    const bool lt = al < ar;
+    const u64 m = lt ? al : ar, M = lt ? ar : al;
+    const u64 twice = m < (0x7feull << 52) ? m + ONE_EXP : m;             // 2 min(|dl|, |dr|)
+    const unsigned eM = static_cast<unsigned>(M >> 52), d = eM - static_cast<unsigned>(m >> 52);
+    const u64 sum = (((M & MANT) | ONE_EXP) << 2) + ((((m & MANT) | ONE_EXP) << 2) >> (d & 3));
+    const unsigned c = static_cast<unsigned>(sum >> 55), sh = 2 + c;      // c: the sum's carry
+    const u64 r = (sum + ((2u << c) - 1) + (static_cast<unsigned>(sum >> sh) & 1u)) >> sh;
+    u64 half = (static_cast<u64>(eM + c - 2) << 52) + r;                  // |dl + dr| / 2
+    half = eM + c >= 2 ? half : 0;
+    const u64 a = d >= 3 || twice < half ? twice : half;
+    return same ? copysign(__longlong_as_double(a), dr) : 0.0;
 }
 
 // CFL signal speed of a cell, sum_d (|u_d| + c) / dx_d, from its momenta m
@@ -244,6 +253,47 @@ __device__ __forceinline__ T signal_speed(const T *m, T rinv, T c, const T (&inv
         sidx += inv_dx[d];
     }
     return fma(rinv, a, c * sidx);
+}
+
+// A double cut to FP32 on the integer pipe (a conversion instruction holds
+// the FP64 pipe like a multiply): relative error below 2^-22; 0 below FP32's
+// normal range, infinity beyond it.
+__device__ __forceinline__ float cut_f32(double x)
+{
+    const unsigned hi = __double2hiint(x), lo = __double2loint(x);
+    const unsigned v = (hi & 0x7fffffffu) - 0x38000000u;   // exponent rebiased, three bits above FP32's place
+    unsigned f = __funnelshift_l(lo, v, 3);
+    f = static_cast<int>(v) < 0x00100000 ? 0u : (v >= 0x0ff00000u ? 0x7f800000u : f);
+    return __uint_as_float(f | (hi & 0x80000000u));
+}
+
+// Whether an FP64 cell's new state u (background rb, pb) is certainly
+// admissible and its CFL signal speed certainly below `below` (or just
+// finite, for below = infinity): an FP32 estimate whose margins, 1e-5 of every
+// term, cover its 2^-22 conversions and rounded operations many times over.
+// The grid's maximum is exact, so a cell below a speed some cell has reached
+// needs no FP64 evaluation; false only means that it has to be evaluated.
+template <int ND>
+__device__ __forceinline__ bool speed_below(const double (&u)[ND + 2], double rb, double pb, float gam,
+                                            const float (&inv_dx)[3], float below)
+{
+    const float r0 = cut_f32(u[0]), rbf = cut_f32(rb), pbf = cut_f32(pb), e = cut_f32(u[ND + 1]);
+    const float r = rbf + r0;
+    const float rinv = __fdividef(1.0f, r);
+    float m2 = 0.0f, adv = 0.0f, sidx = 0.0f;
+#pragma unroll
+    for (int d = 0; d < ND; ++d) {
+        const float m = fabsf(cut_f32(u[1 + d]));
+        m2 = fmaf(m, m, m2);
+        adv = fmaf(m, inv_dx[d], adv);
+        sidx += inv_dx[d];
+    }
+    const float k = 0.5f * m2 * rinv;
+    const float p = pbf + (gam - 1.0f) * (e - k);
+    const float slack = 1e-5f * (fabsf(pbf) + gam * (fabsf(e) + k));
+    const float c2 = gam * (p + slack) * rinv;
+    const float s = 1.00001f * fmaf(adv, rinv, c2 * rsqrtf(c2) * sidx);
+    return r > 0.25f * (fabsf(rbf) + fabsf(r0)) && r < 1e30f && p > slack && s < below;
 }
 
 // Background seen by one cell in HSE mode (all zero in plain mode).
@@ -681,6 +731,7 @@ __device__ __forceinline__ void finish_step(double smax_cta, bool bad_cta, const
         C->max_speed = m;
         C->dt_next = m > 0.0 ? a.cfl / m : 0.0;
         C->counter = 0u;
+        C->reached = 0;
         __threadfence();
     }
 }

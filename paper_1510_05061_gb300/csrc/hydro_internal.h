@@ -21,7 +21,7 @@ struct __align__(16) Ctrl {
     unsigned int counter;   // last-CTA arrival counter (returns to 0)
     int err;            // committed error bits (changed only at finalisation)
     int err_new;        // error bits raised by CTAs of the running step
-    int pad0;
+    int reached;        // FP32 bits of a signal speed the running step's cells have reached (returns to 0)
     double totals[5];   // last conserved-total reduction
     double pad[2];
 };

@@ -523,6 +523,13 @@ __device__ __forceinline__ void step3d_body(const StepArgs &a, int tile, int z0,
     const bool own = gx < nx && gy < ny;
     const int own_off = gy * nx + gx;   // the thread's cell within a plane
 
+    // FP64: a signal speed (FP32 bits, rounded down) that some cell of the
+    // step has reached; cells certainly below it are not evaluated in FP64
+    // (13 FP64 instructions each)
+    constexpr bool PRUNE = sizeof(T) == 8;
+    __shared__ int s_reached;
+    if (PRUNE && tid == 0) s_reached = *const_cast<volatile int *>(&a.ctrl->reached);
+
     // planes z0-H .. z0+LEAD-2 before the march; iteration p stages p+LEAD
     for (int pz = z0 - H; pz <= z0 + LEAD - 2; ++pz) {
         if constexpr (ASYNC) {
@@ -818,17 +825,33 @@ __device__ __forceinline__ void step3d_body(const StepArgs &a, int tile, int z0,
             }
 #pragma unroll
             for (int q = 0; q < NV; ++q) Un[c + q * vs] = u[q];
-            // CFL signal speed and admissibility of the new state
-            const T rho = HSE ? bgR + u[0] : u[0];
-            const T rinv = rcp_t(rho);
-            const T pp = (gam - T(1)) * (u[4] - half_nonneg(u[1] * u[1] + u[2] * u[2] + u[3] * u[3]) * rinv);
-            const T pres = HSE ? bgP + pp : pp;
-            const T gp = gam * pres;
-            const T cs = gp * rsqrt_t(gp * rho);
-            const T s = signal_speed<T, 3>(u + 1, rinv, cs, inv_dx);
-            if (!positive(rho) || !positive(pres) || !isfinite(s)) bad = true;
-            else smax = max_t(smax, s);
+            // CFL signal speed and admissibility of the new state (FP64: of the
+            // cells that could raise the maximum the CTA knows)
+            bool skip = false;
+            if constexpr (PRUNE)
+                skip = speed_below<3>(u, HSE ? double(bgR) : 0.0, HSE ? double(bgP) : 0.0, a.gamma_f, a.inv_dx_f,
+                                      ST == STAGE_RK1 ? INFINITY : __int_as_float(*const_cast<volatile int *>(&s_reached)));
+            if (!skip) {
+                const T rho = HSE ? bgR + u[0] : u[0];
+                const T rinv = rcp_t(rho);
+                const T pp = (gam - T(1)) * (u[4] - half_nonneg(u[1] * u[1] + u[2] * u[2] + u[3] * u[3]) * rinv);
+                const T pres = HSE ? bgP + pp : pp;
+                const T gp = gam * pres;
+                const T cs = gp * rsqrt_t(gp * rho);
+                const T s = signal_speed<T, 3>(u + 1, rinv, cs, inv_dx);
+                if (!positive(rho) || !positive(pres) || !isfinite(s)) bad = true;
+                else if (!PRUNE) smax = max_t(smax, s);
+                else if (s > smax) {
+                    smax = s;
+                    if constexpr (PRUNE && ST != STAGE_RK1) atomicMax(&s_reached, __float_as_int(__double2float_rd(s)));
+                }
+            }
         }
+        // the maximum reached is shared with the other CTAs after the piece's
+        // first planes; later planes rarely raise it
+        if constexpr (PRUNE && ST != STAGE_RK1)
+            if (tid == 0 && p > z0 && p <= z0 + 2)
+                atomicMax(&s_reached, atomicMax(&a.ctrl->reached, *const_cast<volatile int *>(&s_reached)));
         if (xy) {
             T dv[NV];
 #pragma unroll

@@ -78,3 +78,31 @@ def test_outside_the_normal_range(env):
     y = run(env, 2, x)
     assert y[0] == np.inf and y[1] == 0.0 and np.isnan(y[4:]).all()
     assert np.allclose(y[2:4], 1.0 / np.sqrt(x[2:4]), rtol=1e-15)
+
+
+@pytest.mark.parametrize("spread", [0, 1, 2, 3, 4, 60])
+def test_mc_slope_bits(env, spread):
+    """The integer slope has the bits of the FP64 formula, for exponent
+    differences on both sides of the shortcut, ties of the rounding and
+    differences from 2^-900 to 2^900."""
+    torch, hy = env
+    rng = np.random.default_rng(20 + spread)
+    n = 1 << 17
+    e = rng.integers(120, 1920, n)
+    d = rng.integers(-spread, spread + 1, n)
+    m = rng.integers(0, 1 << 52, (2, n), dtype=np.uint64)
+    m[:, : n // 4] &= np.uint64(0xFFFFFFFFFFF00)
+    m[:, n // 4: n // 3] |= np.uint64(0xFFFFFFFFFFF00)
+    m[1, n // 3: n // 2] = m[0, n // 3: n // 2] ^ rng.integers(0, 8, n // 2 - n // 3, dtype=np.uint64)
+    x = ((e.astype(np.uint64) << np.uint64(52)) | m[0]).view(np.float64)
+    y = (((e + d).astype(np.uint64) << np.uint64(52)) | m[1]).view(np.float64)
+    s = rng.choice([-1.0, 1.0], n)
+    x, y = x * s, y * s
+    y[::9] *= -1
+    y[::17] = 0.0
+    xd, yd = (torch.as_tensor(v, device="cuda") for v in (x, y))
+    out = torch.empty_like(xd)
+    hy.hydro_selftest_math(3, xd.data_ptr(), yd.data_ptr(), out.data_ptr(), n, torch.cuda.current_stream().cuda_stream)
+    a = np.minimum(np.minimum(2 * np.abs(x), 2 * np.abs(y)), 0.5 * np.abs(x + y))
+    want = np.where((np.sign(x) * np.sign(y)) > 0, np.copysign(a, y), 0.0)
+    assert np.array_equal(out.cpu().numpy(), want)
