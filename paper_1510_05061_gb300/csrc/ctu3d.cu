@@ -1,6 +1,6 @@
 // ctu3d.cu -- FP64 and FP32 instantiations of the fused 3D corner transport
 // upwind step.  Tiles: FP32 16 x 16 (256 threads, 152 KB of shared memory),
-// FP64 16 x 8 (128 threads, 171 KB); FP32 z-chunks sized for several waves
+// FP64 16 x 8 (256 threads, 171 KB); FP32 z-chunks sized for several waves
 // of the 152 SMs (one CTA per SM), FP64 the balanced grid.
 #include <algorithm>
 
@@ -24,14 +24,15 @@ int ctu_zchunk(const int n[3], bool fp32)
     return (int)((n[2] + nch - 1) / nch);
 }
 
-template <typename T, bool HSE, int TX, int TY>
+template <typename T, bool HSE, int TX, int TY, bool GZ>
 cudaError_t launch_ctu(const StepArgs &a0, cudaStream_t s)
 {
-    auto k = ctu3d_kernel<T, HSE, TX, TY>;
+    auto k = ctu3d_kernel<T, HSE, TX, TY, GZ>;
+    constexpr int NT = CTU3D_THREADS<T, TX, TY>;
     constexpr size_t smem = Ctu3DSmem<T, TX, TY>::bytes;
     static PerDeviceInt resident;   // resident CTAs of the balanced grid, per device
     int g = 0;
-    const cudaError_t e = persistent_grid(resident, k, smem, TX * TY, &g);
+    const cudaError_t e = persistent_grid(resident, k, smem, NT, &g);
     if (e != cudaSuccess) return e;
     StepArgs a = a0;
     a.tiles_x = (a.n[0] + TX - 1) / TX;
@@ -42,11 +43,11 @@ cudaError_t launch_ctu(const StepArgs &a0, cudaStream_t s)
         // marched at the same heights keep their halo rows in L2
         a.zchunk = 0;
         const long long W = (long long)a.tiles_x * ((a.n[1] + TY - 1) / TY) * a.n[2];
-        k<<<(int)std::min<long long>(g, W), TX * TY, smem, s>>>(a);
+        k<<<(int)std::min<long long>(g, W), NT, smem, s>>>(a);
     } else {
         a.zchunk = ctu_zchunk(a.n, sizeof(T) == 4);
         const dim3 grid(a.tiles_x * ((a.n[1] + TY - 1) / TY), (a.n[2] + a.zchunk - 1) / a.zchunk);
-        k<<<grid, TX * TY, smem, s>>>(a);
+        k<<<grid, NT, smem, s>>>(a);
     }
     return cudaGetLastError();
 }
@@ -61,8 +62,12 @@ long long ctu3d_blocks(const int n[3], bool fp32)
 
 cudaError_t launch_ctu3d(const StepArgs &a, cudaStream_t s, bool fp32, bool hse)
 {
-    if (hse) return fp32 ? launch_ctu<float, true, 16, 16>(a, s) : launch_ctu<double, true, 16, 8>(a, s);
-    return fp32 ? launch_ctu<float, false, 16, 16>(a, s) : launch_ctu<double, false, 16, 8>(a, s);
+    // FP64: gravity along z only (always so with the background) leaves out the
+    // x and y gravity terms, whose additions of zero are not folded
+    if (fp32) return hse ? launch_ctu<float, true, 16, 16, false>(a, s) : launch_ctu<float, false, 16, 16, false>(a, s);
+    if (hse) return launch_ctu<double, true, 16, 8, true>(a, s);
+    if (a.grav[0] == 0.0 && a.grav[1] == 0.0) return launch_ctu<double, false, 16, 8, true>(a, s);
+    return launch_ctu<double, false, 16, 8, false>(a, s);
 }
 
 }  // namespace hydro

@@ -122,11 +122,50 @@ __device__ __forceinline__ void predict_axis_bg(const T (&w)[5], const T (&dwd)[
     for (int q = 0; q < 5; ++q) wd[q] = w[q] + hdt * r[q];
 }
 
-template <typename T, bool HSE, int TX, int TY>
+// FP64 predictor along axis d, the one-dimensional A_d terms with hdt / dx_d
+// folded into the coefficients k = hdt / dx_d of u_d, rho, 1/rho and gamma p
+// (16 FP64 instructions per axis where the separate rate and its scaling take
+// 24, one rounding fewer per component).  gh = hdt g; GZ: gravity along z only,
+// whose x and y terms are left out.
+template <bool HSE, bool GZ>
+__device__ __forceinline__ void predict_axis_f64(const double (&w)[5], const double (&dwd)[5], int d, double k, double rinv,
+                                                 double gp, const double (&gh)[3], double hdt, const CellBG<double> &bg,
+                                                 double (&wd)[5])
+{
+    const double rho = HSE ? bg.rho + w[0] : w[0];
+    const double uk = mul_rn(w[1 + d], k);
+    double t0 = fma_rn(uk, dwd[0], mul_rn(mul_rn(rho, k), dwd[1 + d]));
+    double t4 = fma_rn(uk, dwd[4], mul_rn(mul_rn(gp, k), dwd[1 + d]));
+    const double tn = fma_rn(uk, dwd[1 + d], mul_rn(mul_rn(rinv, k), dwd[4]));
+    if (HSE && d == 2) {
+        t0 = fma_rn(uk, bg.drho, t0);
+        t4 = fma_rn(uk, bg.dp, t4);
+    }
+    wd[0] = w[0] - t0;
+    wd[4] = w[4] - t4;
+    const double rr = HSE && d == 2 ? mul_rn(w[0], rinv) : 1.0;
+#pragma unroll
+    for (int e = 0; e < 3; ++e) {
+        wd[1 + e] = e == d ? w[1 + e] - tn : fma_rn(-uk, dwd[1 + e], w[1 + e]);
+        if (!GZ || e == 2) wd[1 + e] = HSE && d == 2 ? fma_rn(gh[e], rr, wd[1 + e]) : wd[1 + e] + gh[e];
+    }
+    if (HSE && d == 2) wd[3] = fma_rn(-mul_rn(hdt, bg.B), rinv, wd[3]);
+}
+
+// FP64 runs 256 threads on its 16 x 8 tile (two warps for each of the SM's
+// four FP64 units instead of one): the loops over ring cells, faces and
+// corrections stride by the CTA's threads, not by the tile's cells, and the
+// faces and the corrections of all three axes form one list each (the axis a
+// run-time value), so that their last, partial warps do not add up.
+template <typename T, int TX, int TY>
+constexpr int CTU3D_THREADS = sizeof(T) == 8 ? 256 : TX * TY;
+
+template <typename T, bool HSE, int TX, int TY, bool GZ>
 __device__ __forceinline__ void ctu3d_body(const StepArgs &a, int tile, int z0, int z1, double dtd,
                                            unsigned char *smem_raw, T &smax, bool &bad)
 {
-    constexpr int ND = 3, NV = 5, NT = TX * TY;
+    constexpr int ND = 3, NV = 5, NT = CTU3D_THREADS<T, TX, TY>;
+    constexpr bool F64 = sizeof(T) == 8;
     using S = Ctu3DSmem<T, TX, TY>;
     constexpr int HX = S::HX, HY = S::HY, EX = S::EX, EY = S::EY;
     T *prim = reinterpret_cast<T *>(smem_raw);
@@ -145,7 +184,8 @@ __device__ __forceinline__ void ctu3d_body(const StepArgs &a, int tile, int z0, 
     const long long vs = a.vstride;
     const int plane = static_cast<int>(a.plane);
     const int gx = x0 + tx, gy = y0 + ty;
-    const bool own = gx < nx && gy < ny;
+    const bool cell = NT == TX * TY || tid < TX * TY;   // the thread has a cell of the tile
+    const bool own = cell && gx < nx && gy < ny;
     const int own_off = gy * nx + gx;
     const T dt = T(dtd), hdt = T(0.5) * T(dtd);
     const T gam = arg_t<T>(a.gamma, a.gamma_f);
@@ -157,6 +197,10 @@ __device__ __forceinline__ void ctu3d_body(const StepArgs &a, int tile, int z0, 
                         arg_t<T>(a.grav[1], a.grav_f[1]),
                         arg_t<T>(a.grav[2], a.grav_f[2])};
     const T hdt_dx[3] = {hdt * inv_dx[0], hdt * inv_dx[1], hdt * inv_dx[2]};   // dt / (2 dx_e)
+    const T gh[3] = {hdt * grav[0], hdt * grav[1], hdt * grav[2]};
+    // FP64: a signal speed some cell of the step has reached (step3d_body)
+    __shared__ int s_reached;
+    if (F64 && tid == 0) s_reached = *const_cast<volatile int *>(&a.ctrl->reached);
 
     auto P = [&](int slot, int q, int hy, int hx) -> T & { return prim[((slot * NV + q) * HY + hy) * HX + hx]; };
     // face-state array arr of plane parity b: 0..5 = x lo, x hi, y lo, y hi,
@@ -222,9 +266,15 @@ __device__ __forceinline__ void ctu3d_body(const StepArgs &a, int tile, int z0, 
             // axis, formed once for the positivity test and stored as faces
             T rp[ND][4];
             bool ok = true;
+            T rinv_c = T(0), gp_c = T(0);
+            if constexpr (F64) {
+                rinv_c = rcp_t(HSE ? bg.rho + w[0] : w[0]);
+                gp_c = gam * (HSE ? bg.p + w[NV - 1] : w[NV - 1]);
+            }
 #pragma unroll
             for (int d = 0; d < ND; ++d) {
-                if constexpr (HSE) predict_axis_bg<T>(w, dw[d], d, hdt, inv_dx[d], gam, grav, bg, wd[d]);
+                if constexpr (F64) predict_axis_f64<HSE, GZ>(w, dw[d], d, hdt_dx[d], rinv_c, gp_c, gh, hdt, bg, wd[d]);
+                else if constexpr (HSE) predict_axis_bg<T>(w, dw[d], d, hdt, inv_dx[d], gam, grav, bg, wd[d]);
                 else predict_axis<T, ND>(w, dw[d], d, hdt, inv_dx[d], gam, grav, wd[d]);
                 rp[d][0] = wd[d][0] - T(0.5) * dw[d][0];
                 rp[d][1] = wd[d][0] + T(0.5) * dw[d][0];
@@ -367,6 +417,92 @@ __device__ __forceinline__ void ctu3d_body(const StepArgs &a, int tile, int z0, 
         }
     };
 
+    // FP64: the faces of all axes through one code path.  any_face: the flux of
+    // the low face along axis ax of cell (cx, cy) of plane pl (parity b),
+    // between array 1, 3 or (z, from the plane of parity bl) zhi and array
+    // 2 ax, into the axis's flux array.
+    constexpr int EN = EY * EX, SX = EY * (TX + 1), SY = (TY + 1) * EX;   // one variable of a state array, of FX, of FY
+    constexpr int OY = 2 * static_cast<int>(S::f1x), OZ = OY + 2 * static_cast<int>(S::f1y);   // FY and FZ behind FX
+    auto any_face = [&](int ax, int pl, int b, int bl, int zhi, int cx, int cy) {
+        if constexpr (F64) {
+            const int right = ((b * 7 + 2 * ax) * NV) * EN + (cy + 1) * EX + cx + 1;
+            const int left = ((bl * 7 + (ax == 2 ? zhi : 2 * ax + 1)) * NV) * EN
+                           + (cy + (ax == 1 ? 0 : 1)) * EX + cx + (ax == 0 ? 0 : 1);
+            const int gf = ax == 0 ? x0 + cx : (ax == 1 ? y0 + cy : pl), n = ax == 0 ? nx : (ax == 1 ? ny : nz);
+            const bool w_lo = gf == 0 && a.bc_lo[ax] == BC_REFLECT, w_hi = gf == n && a.bc_hi[ax] == BC_REFLECT;
+            T wl[NV], wr[NV], f[NV];
+#pragma unroll
+            for (int q = 0; q < NV; ++q) {
+                const T vl = sets[left + q * EN], vr = sets[right + q * EN];
+                const bool flip = q == 1 + ax;
+                wl[q] = w_lo ? (flip ? -vr : vr) : vl;
+                wr[q] = w_hi ? (flip ? -vl : vl) : vr;
+            }
+            T rb = T(0), pb = T(0);
+            if constexpr (HSE) {
+                rb = ax == 2 ? bgT[pl + 2].rho_f : bgT[pl + 2].rho_c;
+                pb = ax == 2 ? bgT[pl + 2].p_f : bgT[pl + 2].p_c;
+            }
+            hllc_f64<ND, HSE>(ax, wl, wr, rb, pb, gam, igm1, f);
+            const int st = ax == 0 ? SX : (ax == 1 ? SY : EN);
+            T *out = f1x + (ax == 0 ? 0 : (ax == 1 ? OY : OZ)) + b * NV * st
+                   + (ax == 0 ? (cy + 1) * (TX + 1) + cx : (ax == 1 ? cy * EX + cx + 1 : (cy + 1) * EX + cx + 1));
+#pragma unroll
+            for (int q = 0; q < NV; ++q) out[q * st] = f[q];
+        }
+    };
+    // any_correct: the transverse correction of the axis-ax states of cell
+    // (cx, cy) (z: of plane p, parity b; x and y: of plane p - 1, parity bm),
+    // as correct() below with each axis's arrays, factors and background.
+    auto any_correct = [&](int ax, int b, int bm, int cx, int cy, const T (&rbz)[2], const T (&pbz)[2], T rbc, T pbc,
+                           T dmz) {
+        if constexpr (F64) {
+            const int c = ax == 2 ? b : bm;
+            const int ix = c * NV * SX + (cy + 1) * (TX + 1) + cx, iy = OY + c * NV * SY + cy * EX + cx + 1;
+            const int iz = OZ + (cy + 1) * EX + cx + 1;
+            // first difference: y fluxes for the x states, x fluxes otherwise;
+            // second: y fluxes for the z states, z fluxes otherwise
+            const int lo1 = ax == 0 ? iy : ix, hi1 = ax == 0 ? iy + EX : ix + 1, st1 = ax == 0 ? SY : SX;
+            const int lo2 = ax == 2 ? iy : iz + bm * NV * EN, hi2 = ax == 2 ? iy + EX : iz + b * NV * EN;
+            const int st2 = ax == 2 ? SY : EN;
+            const T k1 = ax == 0 ? hdt_dx[1] : hdt_dx[0], k2 = ax == 2 ? hdt_dx[1] : hdt_dx[2];
+            T du[NV];
+#pragma unroll
+            for (int q = 0; q < NV; ++q)
+                du[q] = fma_rn(k2, f1x[hi2 + q * st2] - f1x[lo2 + q * st2], mul_rn(k1, f1x[hi1 + q * st1] - f1x[lo1 + q * st1]));
+            if (HSE && ax != 2) du[3] = du[3] + dmz;
+            T *st = sets + ((c * 7 + 2 * ax) * NV) * EN + (cy + 1) * EX + cx + 1;
+            T *dhi = ax == 2 ? st + 2 * NV * EN : st + NV * EN;
+            T wc[2][NV];
+            bool ok = true;
+#pragma unroll
+            for (int s = 0; s < 2; ++s) {
+                T w[NV];
+#pragma unroll
+                for (int q = 0; q < NV; ++q) w[q] = st[(s * NV + q) * EN];
+                const T rb = HSE ? (ax == 2 ? rbz[s] : rbc) : T(0);
+                const T rho = HSE ? rb + w[0] : w[0];
+                const T ke = fma_rn(w[3], w[3], fma_rn(w[2], w[2], mul_rn(w[1], w[1])));
+                const T m[3] = {fma_rn(rho, w[1], -du[1]), fma_rn(rho, w[2], -du[2]), fma_rn(rho, w[3], -du[3])};
+                const T e = fma_rn(w[4], igm1, mul_rn(rho, half_nonneg(ke))) - du[4];
+                wc[s][0] = w[0] - du[0];
+                const T rinv = rcp_t(HSE ? rb + wc[s][0] : wc[s][0]);
+                const T u[3] = {mul_rn(m[0], rinv), mul_rn(m[1], rinv), mul_rn(m[2], rinv)};
+#pragma unroll
+                for (int e1 = 0; e1 < 3; ++e1) wc[s][1 + e1] = u[e1];
+                wc[s][4] = pressure_of<T, 3>(m, u, e, gam - T(1));
+                ok = ok && positive(HSE ? rb + wc[s][0] : wc[s][0])
+                        && positive(HSE ? (ax == 2 ? pbz[s] : pbc) + wc[s][4] : wc[s][4]);
+            }
+#pragma unroll
+            for (int q = 0; q < NV; ++q) {
+                const T hi = st[(NV + q) * EN];
+                if (ok) st[q * EN] = wc[0][q];
+                dhi[q * EN] = ok ? wc[1][q] : hi;
+            }
+        }
+    };
+
     smax = T(0);
     bad = false;
     T fz_prev[NV];
@@ -384,27 +520,37 @@ __device__ __forceinline__ void ctu3d_body(const StepArgs &a, int tile, int z0, 
         __syncthreads();
 
         // 3. first-pass fluxes of plane p, and of the z faces below it
-        for (int i = tid; i < (TX + 1) * EY; i += NT) {
-            const int fi = i % (TX + 1), cy = i / (TX + 1) - 1;
-            T f[NV];
-            x_face(b, p, cy, fi, f);
-#pragma unroll
-            for (int q = 0; q < NV; ++q) FX(b, q, cy, fi) = f[q];
-        }
-        for (int i = rotated_start<NT>(tid); i < EX * (TY + 1); i += NT) {   // second pass off warp 0
-            const int cx = i % EX - 1, fj = i / EX;
-            T f[NV];
-            y_face(b, p, fj, cx, f);
-#pragma unroll
-            for (int q = 0; q < NV; ++q) FY(b, q, fj, cx) = f[q];
-        }
-        if (p >= z0) {
-            for (int i = tid; i < EX * EY; i += NT) {
-                const int cx = i % EX - 1, cy = i / EX - 1;
+        if constexpr (F64) {
+            constexpr int NFX = (TX + 1) * EY, NFY = EX * (TY + 1), NFZ = EX * EY;
+            const int nf = p >= z0 ? NFX + NFY + NFZ : NFX + NFY;
+            for (int i = tid; i < nf; i += NT) {
+                const int ax = i < NFX ? 0 : (i < NFX + NFY ? 1 : 2);
+                const int j = i - (ax == 0 ? 0 : (ax == 1 ? NFX : NFX + NFY)), w = ax == 0 ? TX + 1 : EX;
+                any_face(ax, p, b, ax == 2 ? bm : b, 5, j % w - (ax == 0 ? 0 : 1), j / w - (ax == 1 ? 0 : 1));
+            }
+        } else {
+            for (int i = tid; i < (TX + 1) * EY; i += NT) {
+                const int fi = i % (TX + 1), cy = i / (TX + 1) - 1;
                 T f[NV];
-                z_face(p, 5, cy, cx, f);
+                x_face(b, p, cy, fi, f);
 #pragma unroll
-                for (int q = 0; q < NV; ++q) FZ(b, q, cy, cx) = f[q];
+                for (int q = 0; q < NV; ++q) FX(b, q, cy, fi) = f[q];
+            }
+            for (int i = rotated_start<NT>(tid); i < EX * (TY + 1); i += NT) {   // second pass off warp 0
+                const int cx = i % EX - 1, fj = i / EX;
+                T f[NV];
+                y_face(b, p, fj, cx, f);
+#pragma unroll
+                for (int q = 0; q < NV; ++q) FY(b, q, fj, cx) = f[q];
+            }
+            if (p >= z0) {
+                for (int i = tid; i < EX * EY; i += NT) {
+                    const int cx = i % EX - 1, cy = i / EX - 1;
+                    T f[NV];
+                    z_face(p, 5, cy, cx, f);
+#pragma unroll
+                    for (int q = 0; q < NV; ++q) FZ(b, q, cy, cx) = f[q];
+                }
             }
         }
         __syncthreads();
@@ -420,45 +566,63 @@ __device__ __forceinline__ void ctu3d_body(const StepArgs &a, int tile, int z0, 
             pbc[0] = pbc[1] = bgT[p + 1].p_c;
             dmz = hdt_dx[2] * bgT[p + 1].dp;
         }
-        for (int i = tid; i < TX * TY; i += NT) {
-            const int cx = i % TX, cy = i / TX;
-            T dx1[NV], dy1[NV];
-#pragma unroll
-            for (int q = 0; q < NV; ++q) {
-                dx1[q] = FX(b, q, cy, cx + 1) - FX(b, q, cy, cx);
-                dy1[q] = FY(b, q, cy + 1, cx) - FY(b, q, cy, cx);
-            }
-            correct(b, 4, 4, 6, cy, cx, dx1, hdt_dx[0], dy1, hdt_dx[1], rbz, pbz, T(0));
-        }
         const bool out_plane = p - 1 >= z0 && p - 1 < z1;   // plane p-1 is completed now
-        if (out_plane) {
-            for (int i = tid; i < EX * TY; i += NT) {        // x states: columns -1..TX, tile rows
-                const int cx = i % EX - 1, cy = i / EX;
-                T dy1[NV], dz1[NV];
-#pragma unroll
-                for (int q = 0; q < NV; ++q) {
-                    dy1[q] = FY(bm, q, cy + 1, cx) - FY(bm, q, cy, cx);
-                    dz1[q] = FZ(b, q, cy, cx) - FZ(bm, q, cy, cx);
-                }
-                correct(bm, 0, 0, 1, cy, cx, dy1, hdt_dx[1], dz1, hdt_dx[2], rbc, pbc, dmz);
+        if constexpr (F64) {
+            constexpr int NCZ = TX * TY, NCX = EX * TY, NCY = TX * EY;
+            const int nc = out_plane ? NCZ + NCX + NCY : NCZ;
+            for (int i = tid; i < nc; i += NT) {
+                const int ax = i < NCZ ? 2 : (i < NCZ + NCX ? 0 : 1);
+                const int j = i - (ax == 2 ? 0 : (ax == 0 ? NCZ : NCZ + NCX)), w = ax == 0 ? EX : TX;
+                any_correct(ax, b, bm, j % w - (ax == 0 ? 1 : 0), j / w - (ax == 1 ? 1 : 0), rbz, pbz, rbc[0], pbc[0], dmz);
             }
-            // y states: tile columns, rows -1..TY (second pass off warp 0)
-            for (int i = rotated_start<NT>(tid); i < TX * EY; i += NT) {
-                const int cx = i % TX, cy = i / TX - 1;
-                T dx1[NV], dz1[NV];
+        } else {
+            for (int i = tid; i < TX * TY; i += NT) {
+                const int cx = i % TX, cy = i / TX;
+                T dx1[NV], dy1[NV];
 #pragma unroll
                 for (int q = 0; q < NV; ++q) {
-                    dx1[q] = FX(bm, q, cy, cx + 1) - FX(bm, q, cy, cx);
-                    dz1[q] = FZ(b, q, cy, cx) - FZ(bm, q, cy, cx);
+                    dx1[q] = FX(b, q, cy, cx + 1) - FX(b, q, cy, cx);
+                    dy1[q] = FY(b, q, cy + 1, cx) - FY(b, q, cy, cx);
                 }
-                correct(bm, 2, 2, 3, cy, cx, dx1, hdt_dx[0], dz1, hdt_dx[2], rbc, pbc, dmz);
+                correct(b, 4, 4, 6, cy, cx, dx1, hdt_dx[0], dy1, hdt_dx[1], rbz, pbz, T(0));
+            }
+            if (out_plane) {
+                for (int i = tid; i < EX * TY; i += NT) {        // x states: columns -1..TX, tile rows
+                    const int cx = i % EX - 1, cy = i / EX;
+                    T dy1[NV], dz1[NV];
+#pragma unroll
+                    for (int q = 0; q < NV; ++q) {
+                        dy1[q] = FY(bm, q, cy + 1, cx) - FY(bm, q, cy, cx);
+                        dz1[q] = FZ(b, q, cy, cx) - FZ(bm, q, cy, cx);
+                    }
+                    correct(bm, 0, 0, 1, cy, cx, dy1, hdt_dx[1], dz1, hdt_dx[2], rbc, pbc, dmz);
+                }
+                // y states: tile columns, rows -1..TY (second pass off warp 0)
+                for (int i = rotated_start<NT>(tid); i < TX * EY; i += NT) {
+                    const int cx = i % TX, cy = i / TX - 1;
+                    T dx1[NV], dz1[NV];
+#pragma unroll
+                    for (int q = 0; q < NV; ++q) {
+                        dx1[q] = FX(bm, q, cy, cx + 1) - FX(bm, q, cy, cx);
+                        dz1[q] = FZ(b, q, cy, cx) - FZ(bm, q, cy, cx);
+                    }
+                    correct(bm, 2, 2, 3, cy, cx, dx1, hdt_dx[0], dz1, hdt_dx[2], rbc, pbc, dmz);
+                }
             }
         }
         __syncthreads();
 
         // 5. final fluxes: x and y faces of plane p-1 (over its first-pass
         // arrays), the z face p-1/2 of the own column
-        if (out_plane) {
+        if constexpr (F64) {
+            // x and y faces from the warps without a cell on
+            constexpr int NFX = (TX + 1) * TY, NFY = TX * (TY + 1);
+            if (out_plane)
+                for (int i = (tid + NT - TX * TY) % NT; i < NFX + NFY; i += NT) {
+                    const int ax = i < NFX ? 0 : 1, j = i - (ax ? NFX : 0), w = ax ? TX : TX + 1;
+                    any_face(ax, p - 1, bm, bm, 6, j % w, j / w);
+                }
+        } else if (out_plane) {
             for (int i = tid; i < (TX + 1) * TY; i += NT) {
                 const int fi = i % (TX + 1), cy = i / (TX + 1);
                 T f[NV];
@@ -475,7 +639,7 @@ __device__ __forceinline__ void ctu3d_body(const StepArgs &a, int tile, int z0, 
             }
         }
         T fz[NV];
-        if (p >= z0) z_face(p, 6, ty, tx, fz);
+        if (p >= z0 && cell) z_face(p, 6, ty, tx, fz);
         __syncthreads();
 
         // update of plane p-1 (MUSCL-Hancock sources; HSE: -B on the z momentum)
@@ -489,7 +653,8 @@ __device__ __forceinline__ void ctu3d_body(const StepArgs &a, int tile, int z0, 
                           + (FY(bm, q, ty + 1, tx) - FY(bm, q, ty, tx)) * inv_dx[1]
                           + (fz[q] - fz_prev[q]) * inv_dx[2]);
             }
-            const T msrc = grav[0] * T(0.5) * (FX(bm, 0, ty, tx) + FX(bm, 0, ty, tx + 1))
+            const T msrc = GZ ? grav[2] * T(0.5) * (fz_prev[0] + fz[0])
+                         : grav[0] * T(0.5) * (FX(bm, 0, ty, tx) + FX(bm, 0, ty, tx + 1))
                          + grav[1] * T(0.5) * (FY(bm, 0, ty, tx) + FY(bm, 0, ty + 1, tx))
                          + grav[2] * T(0.5) * (fz_prev[0] + fz[0]);
             const T r_old = u[0];
@@ -498,6 +663,10 @@ __device__ __forceinline__ void ctu3d_body(const StepArgs &a, int tile, int z0, 
             const T rsum = r_old + r_new;   // (the half is folded into g / 2)
 #pragma unroll
             for (int d = 0; d < ND; ++d) {
+                if (GZ && d < 2) {
+                    u[1 + d] += dt * du[1 + d];
+                    continue;
+                }
                 T src = (T(0.5) * grav[d]) * rsum;
                 if (HSE && d == 2) src -= bgT[p + 1].B;
                 u[1 + d] += dt * (du[1 + d] + src);
@@ -505,16 +674,29 @@ __device__ __forceinline__ void ctu3d_body(const StepArgs &a, int tile, int z0, 
             u[4] += dt * (du[4] + msrc);
 #pragma unroll
             for (int q = 0; q < NV; ++q) Un[c + q * vs] = u[q];
-            const T rho = HSE ? bgT[p + 1].rho_c + u[0] : u[0];
-            const T rinv = rcp_t(rho);
-            const T pp = (gam - T(1)) * (u[4] - half_nonneg(u[1] * u[1] + u[2] * u[2] + u[3] * u[3]) * rinv);
-            const T pres = HSE ? bgT[p + 1].p_c + pp : pp;
-            const T gp = gam * pres;
-            const T cs = gp * rsqrt_t(gp * rho);
-            const T s = signal_speed<T, 3>(u + 1, rinv, cs, inv_dx);
-            if (!positive(rho) || !positive(pres) || !isfinite(s)) bad = true;
-            else smax = max_t(smax, s);
+            bool skip = false;
+            if constexpr (F64)
+                skip = speed_below<3>(u, HSE ? double(bgT[p + 1].rho_c) : 0.0, HSE ? double(bgT[p + 1].p_c) : 0.0,
+                                      a.gamma_f, a.inv_dx_f, __int_as_float(*const_cast<volatile int *>(&s_reached)));
+            if (!skip) {
+                const T rho = HSE ? bgT[p + 1].rho_c + u[0] : u[0];
+                const T rinv = rcp_t(rho);
+                const T pp = (gam - T(1)) * (u[4] - half_nonneg(u[1] * u[1] + u[2] * u[2] + u[3] * u[3]) * rinv);
+                const T pres = HSE ? bgT[p + 1].p_c + pp : pp;
+                const T gp = gam * pres;
+                const T cs = gp * rsqrt_t(gp * rho);
+                const T s = signal_speed<T, 3>(u + 1, rinv, cs, inv_dx);
+                if (!positive(rho) || !positive(pres) || !isfinite(s)) bad = true;
+                else if (!F64) smax = max_t(smax, s);
+                else if (s > smax) {
+                    smax = s;
+                    if constexpr (F64) atomicMax(&s_reached, __float_as_int(__double2float_rd(s)));
+                }
+            }
         }
+        if constexpr (F64)
+            if (tid == 0 && p > z0 && p <= z0 + 2)
+                atomicMax(&s_reached, atomicMax(&a.ctrl->reached, *const_cast<volatile int *>(&s_reached)));
         if (p >= z0) {
 #pragma unroll
             for (int q = 0; q < NV; ++q) fz_prev[q] = fz[q];
@@ -522,10 +704,10 @@ __device__ __forceinline__ void ctu3d_body(const StepArgs &a, int tile, int z0, 
     }
 }
 
-template <typename T, bool HSE, int TX, int TY>
-__global__ void __launch_bounds__(TX * TY) ctu3d_kernel(const StepArgs a)
+template <typename T, bool HSE, int TX, int TY, bool GZ>
+__global__ void __launch_bounds__(CTU3D_THREADS<T, TX, TY>) ctu3d_kernel(const StepArgs a)
 {
-    constexpr int NT = TX * TY;
+    constexpr int NT = CTU3D_THREADS<T, TX, TY>;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ double red[32];
     __shared__ int s_last;
@@ -548,7 +730,7 @@ __global__ void __launch_bounds__(TX * TY) ctu3d_kernel(const StepArgs a)
         first = false;
         T sm;
         bool bd;
-        ctu3d_body<T, HSE, TX, TY>(a, t, z0, z1, dtd, smem_raw, sm, bd);
+        ctu3d_body<T, HSE, TX, TY, GZ>(a, t, z0, z1, dtd, smem_raw, sm, bd);
         smax = max_t(smax, sm);
         bad = bad || bd;
     }

@@ -511,16 +511,25 @@ __device__ __forceinline__ void ppm_faces(T am, T a, T ap, T sm, T s, T sp, T &l
 // over random states against 128 bits: mass 4.3e-17, energy 2.6e-16 for both;
 // forming the star state itself takes 33, at 1.3 and 1.8 times that error).
 // Every rounding is spelled out, so that each kernel gives the same bits.
-template <int ND, int D, bool HSE>
-__device__ __forceinline__ void hllc_f64(const double (&wl)[ND + 2], const double (&wr)[ND + 2], double rb, double pb,
-                                         double gam, double igm1, double (&f)[ND + 2])
+// The axis is an argument: a run-time axis (kernels whose warps mix faces of
+// several axes) costs a few selects, no FP64 instruction, and gives the same
+// bits.
+template <int ND, bool HSE>
+__device__ __forceinline__ void hllc_f64(int axis, const double (&wl)[ND + 2], const double (&wr)[ND + 2],
+                                         double rb, double pb, double gam, double igm1, double (&f)[ND + 2])
 {
     constexpr int NV = ND + 2;
     const double rl = HSE ? rb + wl[0] : wl[0];
     const double rr = HSE ? rb + wr[0] : wr[0];
     const double pl = HSE ? pb + wl[NV - 1] : wl[NV - 1];
     const double pr = HSE ? pb + wr[NV - 1] : wr[NV - 1];
-    const double ul = wl[1 + D], ur = wr[1 + D];
+    const auto normal = [&](const double *v) {
+        double n = v[0];
+#pragma unroll
+        for (int e = 1; e < ND; ++e) n = axis == e ? v[e] : n;
+        return n;
+    };
+    const double ul = normal(wl + 1), ur = normal(wr + 1);
     const double gpl = mul_rn(gam, pl), gpr = mul_rn(gam, pr);
     const double cl = mul_rn(gpl, rsqrt_t(mul_rn(gpl, rl)));
     const double cr = mul_rn(gpr, rsqrt_t(mul_rn(gpr, rr)));
@@ -550,17 +559,18 @@ __device__ __forceinline__ void hllc_f64(const double (&wl)[ND + 2], const doubl
     double vk[ND];
 #pragma unroll
     for (int e = 0; e < ND; ++e) vk[e] = left ? wl[1 + e] : wr[1 + e];
+    const double uk = left ? ul : ur;
     double ke = mul_rn(vk[0], vk[0]);
 #pragma unroll
     for (int e = 1; e < ND; ++e) ke = fma_rn(vk[e], vk[e], ke);
     // E_K + p_K = p_K gamma / (gamma - 1) + rho_K |v_K|^2 / 2
     const double hk = fma_rn(pk, igm1 + 1.0, mul_rn(rk, half_nonneg(ke)));
-    const double hs = mul_rn(sstar - vk[D], mul_rn(sk, rcp_t(sk - sstar)));
+    const double hs = mul_rn(sstar - uk, mul_rn(sk, rcp_t(sk - sstar)));
     const double h = star ? hs : 0.0;
-    const double uh = vk[D] + h, g = mul_rn(mk, h);
+    const double uh = uk + h, g = mul_rn(mk, h), pg = ppk + g;
     f[0] = mul_rn(rk, uh);
 #pragma unroll
-    for (int e = 0; e < ND; ++e) f[1 + e] = (e == D) ? fma_rn(f[0], vk[D], ppk + g) : mul_rn(f[0], vk[e]);
+    for (int e = 0; e < ND; ++e) f[1 + e] = fma_rn(f[0], vk[e], axis == e ? pg : 0.0);
     f[NV - 1] = fma_rn(hk, uh, mul_rn(g, sstar));
 }
 
@@ -637,7 +647,7 @@ template <typename T, int ND, int D, bool HSE>
 __device__ __forceinline__ void hllc(const T (&wl)[ND + 2], const T (&wr)[ND + 2], T rb, T pb, T gam, T igm1,
                                      T (&f)[ND + 2])
 {
-    if constexpr (sizeof(T) == 8) hllc_f64<ND, D, HSE>(wl, wr, rb, pb, gam, igm1, f);
+    if constexpr (sizeof(T) == 8) hllc_f64<ND, HSE>(D, wl, wr, rb, pb, gam, igm1, f);
     else hllc_f32<ND, D, HSE>(wl, wr, rb, pb, gam, igm1, f);
 }
 

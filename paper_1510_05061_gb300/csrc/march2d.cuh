@@ -98,6 +98,11 @@ __device__ __forceinline__ void march2d_body(const StepArgs &a, int strip, int r
     smax = T(0);
     bad = false;
 
+    // FP64: a signal speed some cell of the step has reached (step3d_body)
+    constexpr bool PRUNE = sizeof(T) == 8;
+    __shared__ int s_reached;
+    if (PRUNE && t == 0) s_reached = *const_cast<volatile int *>(&a.ctrl->reached);
+
     load(r0 - 2, raw);
     convert(raw, wn);
     load(r0 - 1, raw);
@@ -213,14 +218,29 @@ __device__ __forceinline__ void march2d_body(const StepArgs &a, int strip, int r
             }
 #pragma unroll
             for (int q = 0; q < NV; ++q) Un[cfin + q * vs] = u[q];
-            const T rinv = rcp_t(u[0]);
-            const T pres = (gam - T(1)) * (u[3] - half_nonneg(u[1] * u[1] + u[2] * u[2]) * rinv);
-            const T gp = gam * pres;
-            const T cs = gp * rsqrt_t(gp * u[0]);
-            const T s = signal_speed<T, 2>(u + 1, rinv, cs, inv_dx);
-            if (!(u[0] > T(0)) || !(pres > T(0)) || !isfinite(s)) bad = true;
-            else smax = max_t(smax, s);
+            // (FP64: only of the cells that could raise the maximum the CTA knows)
+            bool skip = false;
+            if constexpr (PRUNE)
+                skip = speed_below<2>(u, 0.0, 0.0, a.gamma_f, a.inv_dx_f,
+                                      ST == STAGE_RK1 ? INFINITY : __int_as_float(*const_cast<volatile int *>(&s_reached)));
+            if (!skip) {
+                const T rinv = rcp_t(u[0]);
+                const T pres = (gam - T(1)) * (u[3] - half_nonneg(u[1] * u[1] + u[2] * u[2]) * rinv);
+                const T gp = gam * pres;
+                const T cs = gp * rsqrt_t(gp * u[0]);
+                const T s = signal_speed<T, 2>(u + 1, rinv, cs, inv_dx);
+                if (!(u[0] > T(0)) || !(pres > T(0)) || !isfinite(s)) bad = true;
+                else if (!PRUNE) smax = max_t(smax, s);
+                else if (s > smax) {
+                    smax = s;
+                    if constexpr (PRUNE && ST != STAGE_RK1) atomicMax(&s_reached, __float_as_int(__double2float_rd(s)));
+                }
+            }
         }
+        // the maximum reached is shared with the other CTAs after the piece's first rows
+        if constexpr (PRUNE && ST != STAGE_RK1)
+            if (t == 0 && p > r0 && p <= r0 + 2)
+                atomicMax(&s_reached, atomicMax(&a.ctrl->reached, *const_cast<volatile int *>(&s_reached)));
         if (xr) {
 #pragma unroll
             for (int q = 0; q < NV; ++q) fxd_prev[q] = fxs[q * NT + tr] - fxv[q];
@@ -239,9 +259,10 @@ __device__ __forceinline__ void march2d_body(const StepArgs &a, int strip, int r
 }
 
 // Resident warps asked of the FP32 kernel: 24 per SM (80 registers; 108
-// registers and 16 warps: 132.6 us at 2048^2, 32 warps with spills: 113).
+// registers and 16 warps: 132.6 us at 2048^2, 32 warps with spills: 113); 12 of
+// the FP64 kernel (168 registers).
 template <typename T, int NT, int ST = STAGE_HANCOCK>
-__global__ void __launch_bounds__(NT, sizeof(T) == 4 ? 768 / NT : 1) march2d_kernel(const StepArgs a)
+__global__ void __launch_bounds__(NT, (sizeof(T) == 4 ? 768 : 384) / NT) march2d_kernel(const StepArgs a)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ double red[32];
