@@ -148,10 +148,12 @@ __device__ __forceinline__ void step2d_body(const StepArgs &a, int tile, double 
         T v[5];
 #pragma unroll
         for (int k = -2; k <= 2; ++k) v[k + 2] = d == 0 ? P(q, hy, hx + k) : P(q, hy + k, hx);
-        const T sm = mc_slope(v[1] - v[0], v[2] - v[1]);
-        const T s0 = mc_slope(v[2] - v[1], v[3] - v[2]);
-        const T sp = mc_slope(v[3] - v[2], v[4] - v[3]);
-        ppm_faces(v[1], v[2], v[3], sm, s0, sp, lo, hi);
+        const T dl = v[2] - v[1], dr = v[3] - v[2];
+        const T sm = mc_slope(v[1] - v[0], dl);
+        const T s0 = mc_slope(dl, dr);
+        const T sp = mc_slope(dr, v[4] - v[3]);
+        if constexpr (sizeof(T) == 8) ppm_limit(v[2], ppm_interface(v[1], v[2], sm, s0), ppm_interface(v[2], v[3], s0, sp), lo, hi);
+        else ppm_faces(v[1], v[2], v[3], sm, s0, sp, lo, hi);
     };
 
     // ---- half step: tile cells, then the cross-shaped ring
