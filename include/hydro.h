@@ -201,9 +201,9 @@ int hydro_set_zchunk(hydro_sim *sim, int zchunk);
 /* Select the 3D tile shape and staging depth: variant index of
    hydro_batch_variant_shape.  Variants 0..3 load each staged plane
    synchronously, 4..7 (the same shapes) copy the next plane asynchronously
-   one plane ahead (MUSCL-Hancock step; the other integrators use the shape
-   only).  Default: chosen from the grid's size and the precision (FP64 mostly
-   variant 6, 16 x 16; FP32 mostly 0, 32 x 8).  Variants 3
+   one plane ahead (FP32 MUSCL-Hancock step; FP64 and the other integrators
+   use the shape only).  Default: chosen from the grid's size and the precision (FP64 mostly
+   variant 2, 16 x 16; FP32 mostly 0, 32 x 8).  Variants 3
    and 7 (32 x 16) are FP32 only.  Results do not depend on the choice
    among 0..7; the paired-cell FP32 variants 8..10 are described below. */
 int hydro_set_tile(hydro_sim *sim, int variant);

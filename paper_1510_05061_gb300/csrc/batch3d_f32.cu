@@ -14,7 +14,7 @@ struct Batch3D {
     {
         static PerDeviceInt cache;   // per device: shared-memory limit and resident grid
         return persistent_grid(cache, step3d_batch_kernel<T, HSE, TX, TY, AS>,
-                               Step3DSmem<T, HSE, TX, TY, RECON_PLM, AS>::bytes, TX * TY, grid);
+                               Step3DSmem<T, HSE, TX, TY, RECON_PLM, AS>::bytes, STEP3D_THREADS<T, TX, TY>, grid);
     }
     static cudaError_t launch(const BatchInst *insts, BatchQueue *q, int parity, int grid, cudaStream_t s)
     {
@@ -22,7 +22,7 @@ struct Batch3D {
         cudaError_t e = ensure(&cap);
         if (e != cudaSuccess) return e;
         step3d_batch_kernel<T, HSE, TX, TY, AS>
-            <<<grid, TX * TY, Step3DSmem<T, HSE, TX, TY, RECON_PLM, AS>::bytes, s>>>(insts, q, parity);
+            <<<grid, STEP3D_THREADS<T, TX, TY>, Step3DSmem<T, HSE, TX, TY, RECON_PLM, AS>::bytes, s>>>(insts, q, parity);
         return cudaGetLastError();
     }
     static int max_grid()

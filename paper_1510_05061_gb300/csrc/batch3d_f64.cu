@@ -8,21 +8,21 @@ namespace hydro {
 
 namespace {
 
-template <typename T, bool HSE, int TX, int TY, bool AS>
+template <typename T, bool HSE, int TX, int TY>
 struct Batch3D {
     static cudaError_t ensure(int *grid)
     {
         static PerDeviceInt cache;   // per device: shared-memory limit and resident grid
-        return persistent_grid(cache, step3d_batch_kernel<T, HSE, TX, TY, AS>,
-                               Step3DSmem<T, HSE, TX, TY, RECON_PLM, AS>::bytes, TX * TY, grid);
+        return persistent_grid(cache, step3d_batch_kernel<T, HSE, TX, TY, false>,
+                               Step3DSmem<T, HSE, TX, TY, RECON_PLM, false>::bytes, STEP3D_THREADS<T, TX, TY>, grid);
     }
     static cudaError_t launch(const BatchInst *insts, BatchQueue *q, int parity, int grid, cudaStream_t s)
     {
         int cap = 0;
         cudaError_t e = ensure(&cap);
         if (e != cudaSuccess) return e;
-        step3d_batch_kernel<T, HSE, TX, TY, AS>
-            <<<grid, TX * TY, Step3DSmem<T, HSE, TX, TY, RECON_PLM, AS>::bytes, s>>>(insts, q, parity);
+        step3d_batch_kernel<T, HSE, TX, TY, false>
+            <<<grid, STEP3D_THREADS<T, TX, TY>, Step3DSmem<T, HSE, TX, TY, RECON_PLM, false>::bytes, s>>>(insts, q, parity);
         return cudaGetLastError();
     }
     static int max_grid()
@@ -35,13 +35,10 @@ struct Batch3D {
 template <bool HSE>
 cudaError_t launch_v(int v, const BatchInst *insts, BatchQueue *q, int parity, int grid, cudaStream_t s)
 {
-    switch (v) {
-    case 0: return Batch3D<double, HSE, 32, 8, false>::launch(insts, q, parity, grid, s);
-    case 1: return Batch3D<double, HSE, 32, 4, false>::launch(insts, q, parity, grid, s);
-    case 2: return Batch3D<double, HSE, 16, 16, false>::launch(insts, q, parity, grid, s);
-    case 4: return Batch3D<double, HSE, 32, 8, true>::launch(insts, q, parity, grid, s);
-    case 5: return Batch3D<double, HSE, 32, 4, true>::launch(insts, q, parity, grid, s);
-    case 6: return Batch3D<double, HSE, 16, 16, true>::launch(insts, q, parity, grid, s);
+    switch (v % 4) {   // helper warps stage in either form: one kernel per shape
+    case 0: return Batch3D<double, HSE, 32, 8>::launch(insts, q, parity, grid, s);
+    case 1: return Batch3D<double, HSE, 32, 4>::launch(insts, q, parity, grid, s);
+    case 2: return Batch3D<double, HSE, 16, 16>::launch(insts, q, parity, grid, s);
     default: return cudaErrorInvalidValue;
     }
 }
@@ -49,13 +46,10 @@ cudaError_t launch_v(int v, const BatchInst *insts, BatchQueue *q, int parity, i
 template <bool HSE>
 int grid_v(int v)
 {
-    switch (v) {
-    case 0: return Batch3D<double, HSE, 32, 8, false>::max_grid();
-    case 1: return Batch3D<double, HSE, 32, 4, false>::max_grid();
-    case 2: return Batch3D<double, HSE, 16, 16, false>::max_grid();
-    case 4: return Batch3D<double, HSE, 32, 8, true>::max_grid();
-    case 5: return Batch3D<double, HSE, 32, 4, true>::max_grid();
-    case 6: return Batch3D<double, HSE, 16, 16, true>::max_grid();
+    switch (v % 4) {   // helper warps stage in either form: one kernel per shape
+    case 0: return Batch3D<double, HSE, 32, 8>::max_grid();
+    case 1: return Batch3D<double, HSE, 32, 4>::max_grid();
+    case 2: return Batch3D<double, HSE, 16, 16>::max_grid();
     default: return 0;
     }
 }

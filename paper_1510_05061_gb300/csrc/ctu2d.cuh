@@ -113,7 +113,7 @@ __device__ __forceinline__ void ctu2d_body(const StepArgs &a, int tile, double d
     const bool own = gx < nx && gy < ny;
     const T dt = T(dtd), hdt = T(0.5) * T(dtd);
     const T gam = arg_t<T>(a.gamma, a.gamma_f);
-    const T igm1 = arg_t<T>(1.0 / (a.gamma - 1.0), a.igm1_f);
+    const T igm1 = arg_t<T>(1.0 / (a.gamma - 1.0), a.igm1_f), sgam = speed_factor<T>(a);
     const T inv_dx[3] = {arg_t<T>(a.inv_dx[0], a.inv_dx_f[0]),
                           arg_t<T>(a.inv_dx[1], a.inv_dx_f[1]),
                           T(0)};
@@ -219,7 +219,7 @@ __device__ __forceinline__ void ctu2d_body(const StepArgs &a, int tile, double d
             wl[q] = w_lo ? (q == 1 ? -xr : xr) : xl;
             wr[q] = w_hi ? (q == 1 ? -xl : xl) : xr;
         }
-        hllc<T, ND, 0, false>(wl, wr, T(0), T(0), gam, igm1, f);
+        hllc<T, ND, 0, false>(wl, wr, T(0), T(0), sgam, igm1, f);
     };
     auto y_flux = [&](const T *sl, const T *sh, int fj, int cx, T (&f)[NV]) {
         const int gf = y0 + fj;
@@ -232,7 +232,7 @@ __device__ __forceinline__ void ctu2d_body(const StepArgs &a, int tile, double d
             wl[q] = w_lo ? (q == 2 ? -yr : yr) : yl;
             wr[q] = w_hi ? (q == 2 ? -yl : yl) : yr;
         }
-        hllc<T, ND, 1, false>(wl, wr, T(0), T(0), gam, igm1, f);
+        hllc<T, ND, 1, false>(wl, wr, T(0), T(0), sgam, igm1, f);
     };
 
     // ---- 3. first-pass fluxes

@@ -189,7 +189,7 @@ __device__ __forceinline__ void ctu3d_body(const StepArgs &a, int tile, int z0, 
     const int own_off = gy * nx + gx;
     const T dt = T(dtd), hdt = T(0.5) * T(dtd);
     const T gam = arg_t<T>(a.gamma, a.gamma_f);
-    const T igm1 = arg_t<T>(1.0 / (a.gamma - 1.0), a.igm1_f);
+    const T igm1 = arg_t<T>(1.0 / (a.gamma - 1.0), a.igm1_f), sgam = speed_factor<T>(a);
     const T inv_dx[3] = {arg_t<T>(a.inv_dx[0], a.inv_dx_f[0]),
                           arg_t<T>(a.inv_dx[1], a.inv_dx_f[1]),
                           arg_t<T>(a.inv_dx[2], a.inv_dx_f[2])};
@@ -341,7 +341,7 @@ __device__ __forceinline__ void ctu3d_body(const StepArgs &a, int tile, int z0, 
             wl[q] = w_lo ? (q == 1 + D ? -vr[q] : vr[q]) : vl[q];
             wr[q] = w_hi ? (q == 1 + D ? -vl[q] : vl[q]) : vr[q];
         }
-        hllc<T, ND, D, HSE>(wl, wr, rb, pb, gam, igm1, f);
+        hllc<T, ND, D, HSE>(wl, wr, rb, pb, sgam, igm1, f);
     };
     using D0 = std::integral_constant<int, 0>;
     using D1 = std::integral_constant<int, 1>;
@@ -443,7 +443,7 @@ __device__ __forceinline__ void ctu3d_body(const StepArgs &a, int tile, int z0, 
                 rb = ax == 2 ? bgT[pl + 2].rho_f : bgT[pl + 2].rho_c;
                 pb = ax == 2 ? bgT[pl + 2].p_f : bgT[pl + 2].p_c;
             }
-            hllc_f64<ND, HSE>(ax, wl, wr, rb, pb, gam, igm1, f);
+            hllc_f64<ND, HSE>(ax, wl, wr, rb, pb, sgam, igm1, f);
             const int st = ax == 0 ? SX : (ax == 1 ? SY : EN);
             T *out = f1x + (ax == 0 ? 0 : (ax == 1 ? OY : OZ)) + b * NV * st
                    + (ax == 0 ? (cy + 1) * (TX + 1) + cx : (ax == 1 ? cy * EX + cx + 1 : (cy + 1) * EX + cx + 1));

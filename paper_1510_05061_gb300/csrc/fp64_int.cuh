@@ -62,12 +62,13 @@ __host__ __device__ __forceinline__ uint64_t rcp_bits(uint64_t b, uint32_t yh)
     return (r >> 10) + (static_cast<uint64_t>(base | (bw & 0x80000000u)) << 32);
 }
 
-// Bits of 1/sqrt(x) for normal positive x; yh: the seed's high word.
-__host__ __device__ __forceinline__ uint64_t rsqrt_bits(uint64_t x, uint32_t yh)
+// 1/sqrt(x) of normal positive x as a mantissa scaled 2^62, to 2^-59, and the
+// word below its binade; yh: the seed's high word.
+__host__ __device__ __forceinline__ uint64_t rsqrt_mantissa(uint64_t x, uint32_t yh, uint32_t &base)
 {
     const uint32_t xl = static_cast<uint32_t>(x), xw = static_cast<uint32_t>(x >> 32);
     const uint32_t xh = (xw & 0xfffffu) | 0x100000u;
-    const uint32_t base = 0x5fd00000u - (((xw + 0x100000u) >> 1) & 0x7ff00000u);
+    base = 0x5fd00000u - (((xw + 0x100000u) >> 1) & 0x7ff00000u);
     const uint32_t my = seed_mantissa(yh, base);
     // odd powers of two: double one factor, so that x y^2 = 2^94 (1 - e)
     const uint32_t odd = (~xw >> 20) & 1u;
@@ -81,10 +82,33 @@ __host__ __device__ __forceinline__ uint64_t rsqrt_bits(uint64_t x, uint32_t yh)
     // e/2 + 3 e^2/8, scaled 2^74
     const int64_t t = static_cast<int64_t>(static_cast<uint64_t>(e) << 11)
                     + static_cast<int64_t>(static_cast<uint64_t>(e2) * 384u);
-    const uint64_t r = ((static_cast<uint64_t>(my) << 42) | 512u)
-                     + static_cast<uint64_t>(static_cast<int64_t>(static_cast<int32_t>(my)) * static_cast<int32_t>(t >> 32))
-                     + umulhi32(my, static_cast<uint32_t>(t));
+    return (static_cast<uint64_t>(my) << 42)
+         + static_cast<uint64_t>(static_cast<int64_t>(static_cast<int32_t>(my)) * static_cast<int32_t>(t >> 32))
+         + umulhi32(my, static_cast<uint32_t>(t));
+}
+
+// Bits of 1/sqrt(x) for normal positive x.
+__host__ __device__ __forceinline__ uint64_t rsqrt_bits(uint64_t x, uint32_t yh)
+{
+    uint32_t base;
+    const uint64_t r = rsqrt_mantissa(x, yh, base) + 512u;
     return (r >> 10) + (static_cast<uint64_t>(base) << 32);
+}
+
+// Bits of k / sqrt(x) for normal positive x and k (bits kb), rounded once: the
+// factor joins before the rounding, a 64 x 64-bit product's upper half (the
+// lowest partial product, below 2^-61, left out).
+__host__ __device__ __forceinline__ uint64_t rsqrt_scaled_bits(uint64_t x, uint32_t yh, uint64_t kb)
+{
+    uint32_t base;
+    const uint64_t r = rsqrt_mantissa(x, yh, base);
+    const uint32_t rh = static_cast<uint32_t>(r >> 32), rl = static_cast<uint32_t>(r);
+    const uint32_t kh = (static_cast<uint32_t>(kb >> 21) & 0x7fffffffu) | 0x80000000u, kl = static_cast<uint32_t>(kb) << 11;
+    uint64_t p = static_cast<uint64_t>(rh) * kh + umulhi32(rh, kl) + umulhi32(rl, kh);   // product of the mantissas, 2^61
+    const bool two = (p >> 62) != 0;                                                   // 2 <= product < 4
+    p = (two ? p : p << 1) + 512u;
+    const uint32_t e = base + (static_cast<uint32_t>(kb >> 32) & 0x7ff00000u) - 0x3ff00000u + (two ? 0x100000u : 0u);
+    return (p >> 10) + (static_cast<uint64_t>(e) << 32);
 }
 
 }  // namespace hydro

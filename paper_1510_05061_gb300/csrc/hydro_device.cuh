@@ -99,6 +99,15 @@ __device__ __forceinline__ double rsqrt_t(double x)
 }
 __device__ __forceinline__ float rsqrt_t(float x) { return rsqrtf(x); }
 
+// k / sqrt(x), k normal and positive, in one rounding and no FP64 instruction.
+__device__ __forceinline__ double scaled_rsqrt(double x, double k)
+{
+    if (static_cast<unsigned>(__double2hiint(x)) - 0x00100000u >= 0x7fe00000u) return k * rsqrt(x);
+    double y;
+    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+    return __longlong_as_double(rsqrt_scaled_bits(__double_as_longlong(x), __double2hiint(y), __double_as_longlong(k)));
+}
+
 // FP64 reciprocal, within 0.53 ulp for every b whose reciprocal is normal;
 // NaN for zero, subnormal, infinite or NaN b, and 0 from 2^1022 on.
 __device__ __forceinline__ double rcp_t(double b)
@@ -133,6 +142,14 @@ __device__ __forceinline__ T pressure_of(const T (&m)[ND], const T (&u)[ND], T e
 #pragma unroll
     for (int d = 1; d < ND; ++d) k = fma_rn(u[d], m[d], k);
     return mul_rn(gm1, fma_rn(T(-0.5), k, e));
+}
+
+// The factor hllc takes for its sound speeds: gamma in FP32, sqrt(gamma) in FP64.
+template <typename T>
+__device__ __forceinline__ T speed_factor(const StepArgs &a)
+{
+    if constexpr (sizeof(T) == 4) return a.gamma_f;
+    else return a.sqrt_gamma;
 }
 
 // A step constant in the kernel's precision: the FP64 value, or its FP32
@@ -533,8 +550,9 @@ __device__ __forceinline__ void ppm_limit(double a, double aL, double aR, double
 // S_R <= 0 -> F_R.  igm1 = 1/(gamma - 1).
 //
 // Arithmetic is arranged to need two square-root reciprocals and two
-// divisions per face: c = g rsqrt(g rho) with g = gamma p.  The star state of
-// Toro eq. (10.39) enters through F*_K = F_K + S_K (U*_K - U_K) and one
+// divisions per face: c = g rsqrt(g rho) with g = gamma p (FP64: p times
+// sqrt(gamma) / sqrt(p rho), the factor joining on the integer pipe).  The
+// star state of Toro eq. (10.39) enters through F*_K = F_K + S_K (U*_K - U_K) and one
 // factor h = S_K (S* - u_K) / (S_K - S*), zero outside the fan:
 //   mass             F_0 = rho_K u_K + rho_K h = rho_K (u_K + h)
 //   tangential       F_0 v_t
@@ -543,17 +561,17 @@ __device__ __forceinline__ void ppm_limit(double a, double aL, double aR, double
 // (S_K (rho*_K - rho_K) = rho_K h; S_K rho_K h = rho_K h u_K + m_K h.)  The
 // star state is never formed, so nothing is subtracted from a nearly equal
 // product, and the fan's branch needs one select (of h) beside those of the
-// side.  36 instructions on the FP64 pipe per face; the same fluxes as
-// separate sums F_K + correction took 44, with the same rounding error (rms
+// side.  33 instructions on the FP64 pipe per face; the same fluxes as
+// separate sums F_K + correction took 44 and the roots and quotients 16 more, with the same rounding error (rms
 // over random states against 128 bits: mass 4.3e-17, energy 2.6e-16 for both;
-// forming the star state itself takes 33, at 1.3 and 1.8 times that error).
+// forming the star state itself saves three more, at 1.3 and 1.8 times that error).
 // Every rounding is spelled out, so that each kernel gives the same bits.
 // The axis is an argument: a run-time axis (kernels whose warps mix faces of
 // several axes) costs a few selects, no FP64 instruction, and gives the same
 // bits.
 template <int ND, bool HSE>
 __device__ __forceinline__ void hllc_f64(int axis, const double (&wl)[ND + 2], const double (&wr)[ND + 2],
-                                         double rb, double pb, double gam, double igm1, double (&f)[ND + 2])
+                                         double rb, double pb, double sgam, double igm1, double (&f)[ND + 2])
 {
     constexpr int NV = ND + 2;
     const double rl = HSE ? rb + wl[0] : wl[0];
@@ -567,15 +585,13 @@ __device__ __forceinline__ void hllc_f64(int axis, const double (&wl)[ND + 2], c
         return n;
     };
     const double ul = normal(wl + 1), ur = normal(wr + 1);
-    const double gpl = mul_rn(gam, pl), gpr = mul_rn(gam, pr);
-    const double cl = mul_rn(gpl, rsqrt_t(mul_rn(gpl, rl)));
-    const double cr = mul_rn(gpr, rsqrt_t(mul_rn(gpr, rr)));
+    const double cl = mul_rn(pl, scaled_rsqrt(mul_rn(pl, rl), sgam));
+    const double cr = mul_rn(pr, scaled_rsqrt(mul_rn(pr, rr), sgam));
     // S_L - u_L = min(-c_L, (u_R - u_L) - c_R) and S_R - u_R = max(c_L - (u_R - u_L), c_R):
-    // the offsets the star factors m_K = rho_K (S_K - u_K) need, and S_L, S_R from them
+    // the offsets the star factors m_K = rho_K (S_K - u_K) need, and the chosen S_K
     const double du = ur - ul;
     const double al = min_t(-cl, du - cr);
     const double ar = max_t(cl - du, cr);
-    const double sl = ul + al, sr = ur + ar;
 
     // Branch-free: every face computes S* and h and the branch of the HLLC
     // fan is applied by selects.  The straight-line code lets a
@@ -584,19 +600,21 @@ __device__ __forceinline__ void hllc_f64(int axis, const double (&wl)[ND + 2], c
     const double dpp = wr[NV - 1] - wl[NV - 1];   // background cancels in the difference
     const double ml = mul_rn(rl, al), mr = mul_rn(rr, ar);
     const double sstar = div_t(fma_rn(-mr, ur, fma_rn(ml, ul, dpp)), ml - mr);
-    const bool sup_l = nonnegative(sl);     // whole fan moves right: F_L
-    const bool sup_r = nonpositive(sr);     // whole fan moves left: F_R
+    // S_L = u_L + a_l >= 0: the whole fan moves right, F_L; S_R = u_R + a_r <= 0:
+    // left, F_R (comparisons of the terms: the rounded sums have these signs)
+    const bool sup_l = order_key(ul) >= order_key(-al);
+    const bool sup_r = order_key(ur) <= order_key(-ar);
     const bool left = sup_l || (!sup_r && nonnegative(sstar));
     const bool star = !sup_l && !sup_r;
     const double rk = left ? rl : rr;
     const double pk = left ? pl : pr;
     const double ppk = left ? wl[NV - 1] : wr[NV - 1];
-    const double sk = left ? sl : sr;
     const double mk = left ? ml : mr;
     double vk[ND];
 #pragma unroll
     for (int e = 0; e < ND; ++e) vk[e] = left ? wl[1 + e] : wr[1 + e];
     const double uk = left ? ul : ur;
+    const double sk = uk + (left ? al : ar);
     double ke = mul_rn(vk[0], vk[0]);
 #pragma unroll
     for (int e = 1; e < ND; ++e) ke = fma_rn(vk[e], vk[e], ke);
@@ -680,12 +698,13 @@ __device__ __forceinline__ void hllc_f32(const float (&wl)[ND + 2], const float 
     f[NV - 1] = star ? fE : f[NV - 1];
 }
 
+// sgam: speed_factor<T>.
 template <typename T, int ND, int D, bool HSE>
-__device__ __forceinline__ void hllc(const T (&wl)[ND + 2], const T (&wr)[ND + 2], T rb, T pb, T gam, T igm1,
+__device__ __forceinline__ void hllc(const T (&wl)[ND + 2], const T (&wr)[ND + 2], T rb, T pb, T sgam, T igm1,
                                      T (&f)[ND + 2])
 {
-    if constexpr (sizeof(T) == 8) hllc_f64<ND, HSE>(D, wl, wr, rb, pb, gam, igm1, f);
-    else hllc_f32<ND, D, HSE>(wl, wr, rb, pb, gam, igm1, f);
+    if constexpr (sizeof(T) == 8) hllc_f64<ND, HSE>(D, wl, wr, rb, pb, sgam, igm1, f);
+    else hllc_f32<ND, D, HSE>(wl, wr, rb, pb, sgam, igm1, f);
 }
 
 // Mirror image of a face state across a wall normal to axis D.

@@ -1,6 +1,7 @@
 // hydro_internal.h -- structures shared by the host API and the kernels.
 #pragma once
 
+#include <cmath>
 #include <cstddef>
 #include <cstdint>
 
@@ -64,12 +65,15 @@ struct StepArgs {
     // redo on the FP64 pipe wherever it rematerialises them
     float gamma_f, igm1_f;
     float inv_dx_f[3], grav_f[3];
+    double sqrt_gamma;  // the FP64 sound speeds' factor (fill_fp32_constants)
 };
 
-// Rounds the FP32 copies of a StepArgs' constants (the same values as a
+// Fills in the constants derived from gamma, 1/dx and g: sqrt(gamma), and the
+// rounded FP32 copies of a StepArgs' constants (the same values as a
 // device-side conversion: IEEE round to nearest of the same doubles).
 inline void fill_fp32_constants(StepArgs &a)
 {
+    a.sqrt_gamma = std::sqrt(a.gamma);
     a.gamma_f = static_cast<float>(a.gamma);
     a.igm1_f = static_cast<float>(1.0 / (a.gamma - 1.0));
     for (int d = 0; d < 3; ++d) {

@@ -59,7 +59,7 @@ __device__ __forceinline__ void march2d_body(const StepArgs &a, int strip, int r
     const long long vs = a.vstride;
     const T dt = T(dtd), hdt = T(0.5) * T(dtd);
     const T gam = arg_t<T>(a.gamma, a.gamma_f);
-    const T igm1 = arg_t<T>(1.0 / (a.gamma - 1.0), a.igm1_f);
+    const T igm1 = arg_t<T>(1.0 / (a.gamma - 1.0), a.igm1_f), sgam = speed_factor<T>(a);
     const T inv_dx[3] = {arg_t<T>(a.inv_dx[0], a.inv_dx_f[0]), arg_t<T>(a.inv_dx[1], a.inv_dx_f[1]), T(0)};
     const T grav[3] = {arg_t<T>(a.grav[0], a.grav_f[0]), arg_t<T>(a.grav[1], a.grav_f[1]), T(0)};
     const CellBG<T> nobg = cell_bg<T, false>(static_cast<const PlaneBGT<T> *>(nullptr), 0);
@@ -184,11 +184,11 @@ __device__ __forceinline__ void march2d_body(const StepArgs &a, int strip, int r
                     wlx[q] = xw_lo ? (q == 1 ? -xlo[q] : xlo[q]) : xl;
                     wrx[q] = xw_hi ? (q == 1 ? -xl : xl) : xlo[q];
                 }
-                hllc<T, ND, 0, false>(wlx, wrx, T(0), T(0), gam, igm1, fxv);
+                hllc<T, ND, 0, false>(wlx, wrx, T(0), T(0), sgam, igm1, fxv);
 #pragma unroll
                 for (int q = 0; q < NV; ++q) fxs[q * NT + t] = fxv[q];
             }
-            if (p >= r0) hllc<T, ND, 1, false>(wl, wr, T(0), T(0), gam, igm1, fy);
+            if (p >= r0) hllc<T, ND, 1, false>(wl, wr, T(0), T(0), sgam, igm1, fy);
             else {
 #pragma unroll
                 for (int q = 0; q < NV; ++q) fy[q] = T(0);

@@ -57,7 +57,7 @@ __device__ __forceinline__ void step2d_body(const StepArgs &a, int tile, double 
     const bool own = gx < nx && gy < ny;
     const T dt = T(dtd), hdt = T(0.5) * T(dtd);
     const T gam = arg_t<T>(a.gamma, a.gamma_f);
-    const T igm1 = arg_t<T>(1.0 / (a.gamma - 1.0), a.igm1_f);
+    const T igm1 = arg_t<T>(1.0 / (a.gamma - 1.0), a.igm1_f), sgam = speed_factor<T>(a);
     const T inv_dx[3] = {arg_t<T>(a.inv_dx[0], a.inv_dx_f[0]),
                           arg_t<T>(a.inv_dx[1], a.inv_dx_f[1]),
                           T(0)};
@@ -242,8 +242,8 @@ __device__ __forceinline__ void step2d_body(const StepArgs &a, int tile, double 
             wly[q] = yw_lo ? (q == 2 ? -yr : yr) : yl;
             wry[q] = yw_hi ? (q == 2 ? -yl : yl) : yr;
         }
-        hllc<T, ND, 0, false>(wlx, wrx, T(0), T(0), gam, igm1, fxv);
-        hllc<T, ND, 1, false>(wly, wry, T(0), T(0), gam, igm1, fyv);
+        hllc<T, ND, 0, false>(wlx, wrx, T(0), T(0), sgam, igm1, fxv);
+        hllc<T, ND, 1, false>(wly, wry, T(0), T(0), sgam, igm1, fyv);
 #pragma unroll
         for (int q = 0; q < NV; ++q) {
             FX(q, ty, tx) = fxv[q];
@@ -261,7 +261,7 @@ __device__ __forceinline__ void step2d_body(const StepArgs &a, int tile, double 
                 wl[q] = WX(wxh, q, r, TX - 1);
                 wr[q] = wall ? (q == 1 ? -wl[q] : wl[q]) : WX(wxl, q, r, TX);
             }
-            hllc<T, ND, 0, false>(wl, wr, T(0), T(0), gam, igm1, f);
+            hllc<T, ND, 0, false>(wl, wr, T(0), T(0), sgam, igm1, f);
 #pragma unroll
             for (int q = 0; q < NV; ++q) FX(q, r, TX) = f[q];
         } else {
@@ -271,7 +271,7 @@ __device__ __forceinline__ void step2d_body(const StepArgs &a, int tile, double 
                 wl[q] = WY(wyh, q, TY - 1, r);
                 wr[q] = wall ? (q == 2 ? -wl[q] : wl[q]) : WY(wyl, q, TY, r);
             }
-            hllc<T, ND, 1, false>(wl, wr, T(0), T(0), gam, igm1, f);
+            hllc<T, ND, 1, false>(wl, wr, T(0), T(0), sgam, igm1, f);
 #pragma unroll
             for (int q = 0; q < NV; ++q) FY(q, TY, r) = f[q];
         }

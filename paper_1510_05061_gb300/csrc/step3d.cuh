@@ -30,10 +30,10 @@
 // asynchronous global->shared copies (cp.async) issued one plane ahead, so
 // that its loads are in flight while the current plane is computed without
 // holding them in registers; without it each plane is loaded, then
-// converted.  The MUSCL-Hancock step offers both (tile variants 4..7 and
-// 0..3) to the autotuner; the other kernels take the precision's default:
-// asynchronous for FP64 (+1.4 % measured on GB300, one CTA per SM), none for
-// FP32 (its further resident CTAs already hide the loads).  The build option
+// converted.  The FP32 MUSCL-Hancock step offers both (tile variants 4..7 and
+// 0..3) to the autotuner, the other FP32 kernels stage synchronously (their
+// further resident CTAs already hide the loads).  FP64 kernels stage from
+// helper warps (STEP3D_HELPERS), in either variant.  The build option
 // HYDRO_ASYNC_STAGING=0 turns the asynchronous path off everywhere.
 #ifndef HYDRO_ASYNC_STAGING
 #define HYDRO_ASYNC_STAGING 1
@@ -59,6 +59,21 @@
 
 namespace hydro {
 
+// FP64: four helper warps beside the tile's cell warps, one for each of the
+// SM's FP64 units.  They stage the planes, form the shared differences, predict
+// the ring and solve the tile's high-side faces, while the cell warps predict,
+// solve and update the tile's own cells; a plane takes two barriers.  With the
+// extra work on the cell warps (two per FP64 unit, 255 registers, three
+// barriers) the step was bound by their latency: FP64 pipe 71 % busy of the 83 %
+// it sustains, and fewer FP64 instructions gained nothing.  With the third
+// warp per unit it is 79 % busy, although the 168 registers left spill (310
+// bytes a plane): RT 256^3 11.30 -> 10.23 ms per step, 101x75x130 1769 -> 1635 us
+// for two, PPM 128^3 4.65 -> 4.18 ms.
+template <typename T>
+constexpr int STEP3D_HELPERS = sizeof(T) == 8 ? 128 : 0;
+template <typename T, int TX, int TY>
+constexpr int STEP3D_THREADS = TX * TY + STEP3D_HELPERS<T>;
+
 template <typename T, bool HSE, int TX, int TY, int RC = RECON_PLM, bool AS = (sizeof(T) == 8)>
 struct Step3DSmem {
     static constexpr int NV = 5;
@@ -77,7 +92,8 @@ struct Step3DSmem {
     // conserved values of the next two planes as copied from HBM, per
     // variable either HY x HX mapped cells or HY rows of TX / W + 2 16-byte
     // vectors (W cells each), whichever is larger, rounded to a vector
-    static constexpr bool async = HYDRO_ASYNC_STAGING != 0 && AS;
+    static constexpr bool helpers = STEP3D_HELPERS<T> > 0;   // stage synchronously, into a spare slot
+    static constexpr bool async = HYDRO_ASYNC_STAGING != 0 && AS && !helpers;
     static constexpr int ctas = HYDRO_STEP3D_MIN_CTAS(T, TX, TY);
     // cells per row vector: 16 bytes, except the FP32 tiles held to 80
     // registers (three CTAs per SM) with synchronous staging, whose four
@@ -159,7 +175,7 @@ template <typename T, bool HSE, int TX, int TY, int ST = STAGE_HANCOCK, int RC =
 __device__ __forceinline__ void step3d_body(const StepArgs &a, int tile, int z0, int z1, double dtd,
                                             unsigned char *smem_raw, T &smax, bool &bad)
 {
-    constexpr int ND = 3, NV = 5, NT = TX * TY;
+    constexpr int ND = 3, NV = 5, NT = TX * TY;   // NT: threads with a cell
     static_assert(RC == RECON_PLM || (ST != STAGE_HANCOCK && !HSE), "PPM: method-of-lines stages, no background");
     static_assert(NT >= 32 + TX && TY <= 32, "high-side faces: x on warp 0, y on warp 1");
     using S = Step3DSmem<T, HSE, TX, TY, RC, AS>;
@@ -170,6 +186,11 @@ __device__ __forceinline__ void step3d_body(const StepArgs &a, int tile, int z0,
     // staging plane p + H and the half step of plane p share one barrier
     // interval; without it H - 1 and a barrier between the two
     constexpr bool MERGED = S::spare;
+    // threads that stage (the helpers, numbered from 0, or all), and whether
+    // this thread has a cell
+    constexpr bool WS = S::helpers;
+    static_assert(!WS || MERGED, "the helpers stage into the spare slot");
+    constexpr int NS = WS ? STEP3D_HELPERS<T> : NT;
     constexpr int LEAD = MERGED ? H : H - 1;
     T *prim = reinterpret_cast<T *>(smem_raw);
     T *wxl = prim + S::prim, *wxh = wxl + S::wx;
@@ -181,6 +202,8 @@ __device__ __forceinline__ void step3d_body(const StepArgs &a, int tile, int z0,
 
     const int nx = a.n[0], ny = a.n[1], nz = a.n[2];
     const int tid = threadIdx.x, tx = tid % TX, ty = tid / TX;
+    const bool cellw = !WS || tid < NT;
+    const int sid = WS ? tid - NT : tid;
     const int x0 = (tile % a.tiles_x) * TX;
     const int y0 = (tile / a.tiles_x) * TY;
     const T *__restrict__ U = static_cast<const T *>(a.U);
@@ -192,7 +215,7 @@ __device__ __forceinline__ void step3d_body(const StepArgs &a, int tile, int z0,
     const int plane = static_cast<int>(a.plane);
     const T dt = T(dtd), hdt = T(0.5) * T(dtd);
     const T gam = arg_t<T>(a.gamma, a.gamma_f);
-    const T igm1 = arg_t<T>(1.0 / (a.gamma - 1.0), a.igm1_f);
+    const T igm1 = arg_t<T>(1.0 / (a.gamma - 1.0), a.igm1_f), sgam = speed_factor<T>(a);
     const PlaneBGT<T> *bgT = static_cast<const PlaneBGT<T> *>(a.bgT);
     const T inv_dx[3] = {arg_t<T>(a.inv_dx[0], a.inv_dx_f[0]),
                           arg_t<T>(a.inv_dx[1], a.inv_dx_f[1]),
@@ -220,12 +243,12 @@ __device__ __forceinline__ void step3d_body(const StepArgs &a, int tile, int z0,
     // the same primitives (the same conversion of the same values).  The
     // x-y mapping of a thread's elements is the same on every plane and is
     // computed once.
-    constexpr int NLOAD = (HX * HY + NT - 1) / NT;
+    constexpr int NLOAD = (HX * HY + NS - 1) / NS;
     constexpr int HXY = HX * HY;
     constexpr int W = S::VW;                  // cells per vector
     constexpr int NQ = TX / W + 2;            // vectors per row
     constexpr int NVEC = NQ * HY;
-    constexpr int NVL = (NVEC + NT - 1) / NT;
+    constexpr int NVL = (NVEC + NS - 1) / NS;
     constexpr int NOFF = NLOAD > NVL ? NLOAD : NVL;
     constexpr int RPS = static_cast<int>(S::rps);
     using V16 = typename RowVec<T, W>::V;
@@ -237,7 +260,7 @@ __device__ __forceinline__ void step3d_body(const StepArgs &a, int tile, int z0,
     if (vec) {
 #pragma unroll
         for (int j = 0; j < NVL; ++j) {
-            const int i = tid + j * NT;
+            const int i = sid + j * NS;
             const int k = i % NQ, hy = i / NQ;
             bool fy = false;
             const int gym = i < NVEC ? map_index(y0 + hy - H, ny, a.bc_lo[1], a.bc_hi[1], fy) : 0;
@@ -247,7 +270,7 @@ __device__ __forceinline__ void step3d_body(const StepArgs &a, int tile, int z0,
     } else {
 #pragma unroll
         for (int j = 0; j < NLOAD; ++j) {
-            const int i = tid + j * NT;
+            const int i = sid + j * NS;
             const int hx = i % HX, hy = i / HX;
             bool fx, fy;
             const int gxm = map_index(x0 + hx - H, nx, a.bc_lo[0], a.bc_hi[0], fx);
@@ -308,7 +331,7 @@ __device__ __forceinline__ void step3d_body(const StepArgs &a, int tile, int z0,
             if (vec) {
 #pragma unroll
                 for (int j = 0; j < NVL; ++j) {
-                    const int i = tid + j * NT;
+                    const int i = sid + j * NS;
                     if (i < NVEC) {
 #pragma unroll
                         for (int q = 0; q < NV; ++q) cp_async_vec<W * sizeof(T)>(rb + q * RPS + i * W, Up + xyoff[j] + q * vs);
@@ -317,7 +340,7 @@ __device__ __forceinline__ void step3d_body(const StepArgs &a, int tile, int z0,
             } else {
 #pragma unroll
                 for (int j = 0; j < NLOAD; ++j) {
-                    const int i = tid + j * NT;
+                    const int i = sid + j * NS;
                     if (i < HXY) {
 #pragma unroll
                         for (int q = 0; q < NV; ++q) cp_async_elem(rb + q * RPS + i, Up + xyoff[j] + q * vs);
@@ -328,7 +351,7 @@ __device__ __forceinline__ void step3d_body(const StepArgs &a, int tile, int z0,
         } else {
 #pragma unroll
             for (int j = 0; j < NLOAD; ++j) {
-                const int i = tid + j * NT;
+                const int i = sid + j * NS;
                 if (i < HXY) {
 #pragma unroll
                     for (int q = 0; q < NV; ++q) raw[ASYNC ? 0 : j][q] = Up[xyoff[j] + q * vs];
@@ -346,7 +369,7 @@ __device__ __forceinline__ void step3d_body(const StepArgs &a, int tile, int z0,
         if (ASYNC && vec) {
 #pragma unroll
             for (int j = 0; j < NVL; ++j) {
-                const int i = tid + j * NT;
+                const int i = sid + j * NS;
                 if (i < NVEC) {
                     V16 rv[NV];
 #pragma unroll
@@ -358,7 +381,7 @@ __device__ __forceinline__ void step3d_body(const StepArgs &a, int tile, int z0,
         }
 #pragma unroll
         for (int j = 0; j < NLOAD; ++j) {
-            const int i = tid + j * NT;
+            const int i = sid + j * NS;
             if (i < HXY) {
                 const int hx = i % HX, hy = i / HX;
                 T v[NV], o[NVS];
@@ -387,12 +410,36 @@ __device__ __forceinline__ void step3d_body(const StepArgs &a, int tile, int z0,
         // their registers would spill)
 #pragma unroll
         for (int j = 0; j < NVL; ++j) {
-            const int i = tid + j * NT;
+            const int i = sid + j * NS;
             if (i < NVEC) {
                 V16 rv[NV];
 #pragma unroll
                 for (int q = 0; q < NV; ++q) rv[q] = ld_vec<T, W>(Up + xyoff[j] + q * vs);
                 put_vec(slot, i, rv, (flips >> (2 * j + 1)) & 1u, fz, rho_bg);
+            }
+        }
+    };
+
+    // the planes before the march (with helpers: by every thread of the CTA, a
+    // few elements of different planes in flight each)
+    auto stage_first = [&](int pz0) {
+        constexpr int NP = H + LEAD - 1, NA = NT + STEP3D_HELPERS<T>, NE = (NP * HXY + NA - 1) / NA;
+#pragma unroll
+        for (int j = 0; j < NE; ++j) {
+            const int i = tid + j * NA;
+            if (i < NP * HXY) {
+                const int pz = pz0 + i / HXY, hx = i % HXY % HX, hy = i % HXY / HX;
+                bool fx, fy, fz;
+                const int gz = map_index<true>(pz, nz, a.bc_lo[2], a.bc_hi[2], fz);
+                const int gym = map_index(y0 + hy - H, ny, a.bc_lo[1], a.bc_hi[1], fy);
+                const int gxm = map_index(x0 + hx - H, nx, a.bc_lo[0], a.bc_hi[0], fx);
+                const T *src = U + (long long)gz * plane + gym * nx + gxm;
+                T v[NV], o[NVS];
+#pragma unroll
+                for (int q = 0; q < NV; ++q) v[q] = src[q * vs];
+                convert(v, fx, fy, fz, HSE ? bgT[pz + 2].rho_c : T(0), o);
+#pragma unroll
+                for (int q = 0; q < NVS; ++q) P((pz + 2 * NR) % NR, q, hy, hx) = o[q];
             }
         }
     };
@@ -410,18 +457,12 @@ __device__ __forceinline__ void step3d_body(const StepArgs &a, int tile, int z0,
     auto DY = [&](int pz, int q, int f, int cx) -> T & {   // f in [-2, TY], cx in [-1, TX]
         return dif[(pz & 1) * (S::dxn + S::dyn) + S::dxn + (q * (TY + 3) + f + 2) * DYR + cx + 1];
     };
-    // Each SM sub-partition (warp mod 4) has its own FP64 unit.  The ring
-    // cells' half steps run on warps 2 and 3 (ring_start below), so the
-    // differences are formed by warps 0, 1, 4, 5, ... (those with warp mod 4
-    // < 2): the four units then carry about the same FP64 work between the
-    // barriers.
-    static_assert(!DIFFS || NT % 128 == 0, "differences on half of the warps");
-    constexpr int NDT = NT / 2;
-    const int dlane = ((tid >> 7) << 6) + (tid & 63);   // index among the difference threads
+    // (formed by the second half of the helpers; the first half predicts the ring)
+    constexpr int NDT = NS / 2;
     auto form_diffs = [&](int pz) {
         const int sl = (pz + 2 * NR) % NR;
-        if (tid & 64) return;
-        for (int i = dlane; i < NDX + NDY; i += NDT) {
+        if (sid < NDT) return;
+        for (int i = sid - NDT; i < NDX + NDY; i += NDT) {
             if (i < NDX) {
                 const int cy = i / DXR - 1, f = i % DXR - 2;
 #pragma unroll
@@ -540,7 +581,7 @@ __device__ __forceinline__ void step3d_body(const StepArgs &a, int tile, int z0,
     smax = T(0);
     bad = false;
     const int gx = x0 + tx, gy = y0 + ty;
-    const bool own = gx < nx && gy < ny;
+    const bool own = cellw && gx < nx && gy < ny;
     const int own_off = gy * nx + gx;   // the thread's cell within a plane
 
     // FP64: a signal speed (FP32 bits, rounded down) that some cell of the
@@ -551,33 +592,37 @@ __device__ __forceinline__ void step3d_body(const StepArgs &a, int tile, int z0,
     if (PRUNE && tid == 0) s_reached = *const_cast<volatile int *>(&a.ctrl->reached);
 
     // planes z0-H .. z0+LEAD-2 before the march; iteration p stages p+LEAD
-    for (int pz = z0 - H; pz <= z0 + LEAD - 2; ++pz) {
-        if constexpr (ASYNC) {
-            fetch(pz);
-            store(pz);
-        } else {
-            stage_sync(pz);
+    if constexpr (WS) {
+        stage_first(z0 - H);
+    } else {
+        for (int pz = z0 - H; pz <= z0 + LEAD - 2; ++pz) {
+            if constexpr (ASYNC) {
+                fetch(pz);
+                store(pz);
+            } else {
+                stage_sync(pz);
+            }
         }
     }
     __syncthreads();
     if constexpr (ASYNC) fetch(z0 + LEAD - 1);
     if constexpr (DIFFS) {
-        form_diffs(z0 - 1);
+        if (!cellw) form_diffs(z0 - 1);
         __syncthreads();
     }
-    if constexpr (OWNZ) {
+    if (OWNZ && cellw) {
         // the own column's z difference below plane z0-1 (planes staged above)
 #pragma unroll
         for (int q = 0; q < NV; ++q)
             dz[q] = P((z0 - 1 + 2 * NR) % NR, q, ty + H, tx + H) - P((z0 - 2 + 2 * NR) % NR, q, ty + H, tx + H);
     }
-    if constexpr (PPMZ) {
+    if (PPMZ && cellw) {
 #pragma unroll
         for (int q = 0; q < NV; ++q) {
             const T a = ppm_up(z0 - 3, q), b = ppm_up(z0 - 2, q), c = ppm_up(z0 - 1, q), d = ppm_up(z0, q);
             pz_d[q] = d - c;
             pz_s[q] = mc_slope(c - b, pz_d[q]);
-            pz_i[q] = ppm_interface(b, c, mc_slope(b - a, c - b), pz_s[q]);
+            if constexpr (PPMZ) pz_i[q] = ppm_interface(b, c, mc_slope(b - a, c - b), pz_s[q]);
         }
     }
     for (int p = z0 - 1; p <= z1; ++p) {
@@ -595,7 +640,7 @@ __device__ __forceinline__ void step3d_body(const StepArgs &a, int tile, int z0,
             // converts the elements it copied itself)
             if (p + LEAD <= z1 + H - 1) store(p + LEAD);
             if (p + LEAD + 1 <= z1 + H - 1) fetch(p + LEAD + 1);
-        } else if (p + LEAD <= z1 + H - 1) {
+        } else if (!WS && p + LEAD <= z1 + H - 1) {   // (the helpers stage beside the faces, below)
             stage_sync(p + LEAD);
         }
         if constexpr (!MERGED) __syncthreads();
@@ -622,7 +667,9 @@ __device__ __forceinline__ void step3d_body(const StepArgs &a, int tile, int z0,
 
         // ---- step 2: half step; own cell first (z faces kept in registers)
         T zlo[NV], ztop[NV];
-        if constexpr (RC == RECON_PPM) {
+        if (!cellw) {
+            // helpers: their part of the plane follows
+        } else if constexpr (RC == RECON_PPM) {
 #pragma unroll
             for (int q = 0; q < NV; ++q) {
                 if constexpr (PPMZ) ppm_own_z(p, q, zlo[q], ztop[q]);
@@ -659,13 +706,12 @@ __device__ __forceinline__ void step3d_body(const StepArgs &a, int tile, int z0,
                 }
             }
         }
-        if (xy) {
+        if (xy && (!WS || (!cellw && sid < (DIFFS ? NS / 2 : NS)))) {
             // ring cells: x = -1 and x = TX (rows 0..TY-1), y = -1 and y = TY
             // (columns 0..TX-1); only their face toward the tile is needed
             constexpr int NRING = 2 * TY + 2 * TX;
-            // (FP64: from warp 2 on, see form_diffs)
-            const int ring_start = DIFFS ? rotated_start<NT>(tid) : tid;
-            for (int i = ring_start; i < NRING; i += NT) {
+            constexpr int NRT = WS ? (DIFFS ? NS / 2 : NS) : NT;
+            for (int i = sid; i < NRING; i += NRT) {
                 int cx, cy;
                 bool xside;
                 if (i < 2 * TY) { xside = true; cy = i >> 1; cx = (i & 1) ? TX : -1; }
@@ -709,7 +755,7 @@ __device__ __forceinline__ void step3d_body(const StepArgs &a, int tile, int z0,
         // the next plane's differences (staged and visible since the last
         // barrier) for the next iteration's half step
         if constexpr (DIFFS)
-            if (p + 1 <= z1) form_diffs(p + 1);
+            if (!cellw && p + 1 <= z1) form_diffs(p + 1);
         __syncthreads();
 
         // ---- step 3: face fluxes.  Each thread evaluates the low x face and
@@ -733,7 +779,62 @@ __device__ __forceinline__ void step3d_body(const StepArgs &a, int tile, int z0,
             }
         };
         T fz[NV];
-        if (xy) {
+        if (WS && !cellw) {
+            // helpers: the tile's high-side x and y faces as one list on the
+            // last warp, and plane p + H into the spare slot (last read by
+            // plane p - 1's half step)
+            if constexpr (WS) {
+                if (xy && sid >= NS - 32)
+                    for (int i = sid - (NS - 32); i < TY + TX; i += 32) {
+                        const bool isx = i < TY;
+                        const int r = isx ? i : i - TY;
+                        const bool wall = isx ? x0 + TX == nx && a.bc_hi[0] == BC_REFLECT
+                                              : y0 + TY == ny && a.bc_hi[1] == BC_REFLECT;
+                        T wl[NV], wr[NV], f[NV];
+#pragma unroll
+                        for (int q = 0; q < NV; ++q) {
+                            const T *l = isx ? &WX(wxh, q, r, TX - 1) : &WY(wyh, q, TY - 1, r);
+                            const T *h = isx ? &WX(wxl, q, r, TX) : &WY(wyl, q, TY, r);
+                            wl[q] = *l;
+                            wr[q] = wall ? (q == (isx ? 1 : 2) ? -wl[q] : wl[q]) : *h;
+                        }
+                        hllc_f64<ND, HSE>(isx ? 0 : 1, wl, wr, rb_c, pb_c, sgam, igm1, f);
+#pragma unroll
+                        for (int q = 0; q < NV; ++q) *(isx ? &FX(q, r, TX) : &FY(q, TY, r)) = f[q];
+                    }
+                if (p + H <= z1 + H - 1) stage_sync(p + H);
+            }
+        } else if (WS && xy) {
+            // one face after the other (three warps per FP64 unit overlap;
+            // the three at once would not fit the cell warps' registers)
+            const bool xw_lo = x0 + tx == 0 && a.bc_lo[0] == BC_REFLECT;
+            const bool xw_hi = x0 + tx == nx && a.bc_hi[0] == BC_REFLECT;
+            const bool yw_lo = y0 + ty == 0 && a.bc_lo[1] == BC_REFLECT;
+            const bool yw_hi = y0 + ty == ny && a.bc_hi[1] == BC_REFLECT;
+            T wl[NV], wr[NV], f[NV];
+            z_states(wl, wr);
+            hllc<T, ND, 2, HSE>(wl, wr, rb_f, pb_f, sgam, igm1, fz);
+            asm volatile("" ::: "memory");
+#pragma unroll
+            for (int q = 0; q < NV; ++q) {
+                const T l = WX(wxh, q, ty, tx - 1), r = WX(wxl, q, ty, tx);
+                wl[q] = xw_lo ? (q == 1 ? -r : r) : l;
+                wr[q] = xw_hi ? (q == 1 ? -l : l) : r;
+            }
+            hllc<T, ND, 0, HSE>(wl, wr, rb_c, pb_c, sgam, igm1, f);
+#pragma unroll
+            for (int q = 0; q < NV; ++q) FX(q, ty, tx) = f[q];
+            asm volatile("" ::: "memory");
+#pragma unroll
+            for (int q = 0; q < NV; ++q) {
+                const T l = WY(wyh, q, ty - 1, tx), r = WY(wyl, q, ty, tx);
+                wl[q] = yw_lo ? (q == 2 ? -r : r) : l;
+                wr[q] = yw_hi ? (q == 2 ? -l : l) : r;
+            }
+            hllc<T, ND, 1, HSE>(wl, wr, rb_c, pb_c, sgam, igm1, f);
+#pragma unroll
+            for (int q = 0; q < NV; ++q) FY(q, ty, tx) = f[q];
+        } else if (xy) {
             T wlx[NV], wrx[NV], wly[NV], wry[NV], wlz[NV], wrz[NV], fxv[NV], fyv[NV];
             // the low face of this cell is a wall when it sits on the domain's
             // low boundary, or on the high boundary (ragged tile: the cell is
@@ -769,9 +870,9 @@ __device__ __forceinline__ void step3d_body(const StepArgs &a, int tile, int z0,
                 }
                 z_states(wlz, wrz);
             }
-            hllc<T, ND, 0, HSE>(wlx, wrx, rb_c, pb_c, gam, igm1, fxv);
-            hllc<T, ND, 1, HSE>(wly, wry, rb_c, pb_c, gam, igm1, fyv);
-            hllc<T, ND, 2, HSE>(wlz, wrz, rb_f, pb_f, gam, igm1, fz);
+            hllc<T, ND, 0, HSE>(wlx, wrx, rb_c, pb_c, sgam, igm1, fxv);
+            hllc<T, ND, 1, HSE>(wly, wry, rb_c, pb_c, sgam, igm1, fyv);
+            hllc<T, ND, 2, HSE>(wlz, wrz, rb_f, pb_f, sgam, igm1, fz);
 #pragma unroll
             for (int q = 0; q < NV; ++q) {
                 FX(q, ty, tx) = fxv[q];
@@ -785,7 +886,7 @@ __device__ __forceinline__ void step3d_body(const StepArgs &a, int tile, int z0,
             // them packed on the first TX + TY threads, which measured faster
             // there (the other form compiled to fewer registers and less ILP).
             constexpr bool split = NT <= 256;
-            if (split ? (tid < TY || (tid >= 32 && tid < 32 + TX)) : tid < TY + TX) {
+            if (!WS && (split ? (tid < TY || (tid >= 32 && tid < 32 + TX)) : tid < TY + TX)) {
                 const bool isx = tid < TY;
                 const int r = isx ? tid : (split ? tid - 32 : tid - TY);
                 T wl[NV], wr[NV], f[NV];
@@ -796,7 +897,7 @@ __device__ __forceinline__ void step3d_body(const StepArgs &a, int tile, int z0,
                         wl[q] = WX(wxh, q, r, TX - 1);
                         wr[q] = wall ? (q == 1 ? -wl[q] : wl[q]) : WX(wxl, q, r, TX);
                     }
-                    hllc<T, ND, 0, HSE>(wl, wr, rb_c, pb_c, gam, igm1, f);
+                    hllc<T, ND, 0, HSE>(wl, wr, rb_c, pb_c, sgam, igm1, f);
 #pragma unroll
                     for (int q = 0; q < NV; ++q) FX(q, r, TX) = f[q];
                 } else {
@@ -806,7 +907,7 @@ __device__ __forceinline__ void step3d_body(const StepArgs &a, int tile, int z0,
                         wl[q] = WY(wyh, q, TY - 1, r);
                         wr[q] = wall ? (q == 2 ? -wl[q] : wl[q]) : WY(wyl, q, TY, r);
                     }
-                    hllc<T, ND, 1, HSE>(wl, wr, rb_c, pb_c, gam, igm1, f);
+                    hllc<T, ND, 1, HSE>(wl, wr, rb_c, pb_c, sgam, igm1, f);
 #pragma unroll
                     for (int q = 0; q < NV; ++q) FY(q, TY, r) = f[q];
                 }
@@ -814,7 +915,7 @@ __device__ __forceinline__ void step3d_body(const StepArgs &a, int tile, int z0,
         } else if (p == z1) {
             T wlz[NV], wrz[NV];
             z_states(wlz, wrz);
-            hllc<T, ND, 2, HSE>(wlz, wrz, rb_f, pb_f, gam, igm1, fz);
+            hllc<T, ND, 2, HSE>(wlz, wrz, rb_f, pb_f, sgam, igm1, fz);
         } else {
 #pragma unroll
             for (int q = 0; q < NV; ++q) fz[q] = T(0);
@@ -884,7 +985,7 @@ __device__ __forceinline__ void step3d_body(const StepArgs &a, int tile, int z0,
         if constexpr (PRUNE && ST != STAGE_RK1)
             if (tid == 0 && p > z0 && p <= z0 + 2)
                 atomicMax(&s_reached, atomicMax(&a.ctrl->reached, *const_cast<volatile int *>(&s_reached)));
-        if (xy) {
+        if (xy && cellw) {
             T dv[NV];
 #pragma unroll
             for (int q = 0; q < NV; ++q)
@@ -904,9 +1005,10 @@ __device__ __forceinline__ void step3d_body(const StepArgs &a, int tile, int z0,
 
 template <typename T, bool HSE, int TX, int TY, int ST = STAGE_HANCOCK, int RC = RECON_PLM,
           bool AS = (sizeof(T) == 8), bool GZ = false>
-__global__ void __launch_bounds__(TX * TY, HYDRO_STEP3D_MIN_CTAS(T, TX, TY)) step3d_kernel(const StepArgs a)
+__global__ void __launch_bounds__(STEP3D_THREADS<T, TX, TY>, HYDRO_STEP3D_MIN_CTAS(T, TX, TY))
+step3d_kernel(const StepArgs a)
 {
-    constexpr int NT = TX * TY;
+    constexpr int NT = STEP3D_THREADS<T, TX, TY>;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ double red[32];
     __shared__ int s_last;
@@ -955,10 +1057,10 @@ __global__ void __launch_bounds__(TX * TY, HYDRO_STEP3D_MIN_CTAS(T, TX, TY)) ste
 // that instance's next dt (per-instance CFL).  A frozen instance (step limit
 // reached, or its error state) is skipped: its state stays where it is.
 template <typename T, bool HSE, int TX, int TY, bool AS = (sizeof(T) == 8)>
-__global__ void __launch_bounds__(TX * TY, HYDRO_STEP3D_MIN_CTAS(T, TX, TY))
+__global__ void __launch_bounds__(STEP3D_THREADS<T, TX, TY>, HYDRO_STEP3D_MIN_CTAS(T, TX, TY))
 step3d_batch_kernel(const BatchInst *__restrict__ insts, BatchQueue *q, int parity)
 {
-    constexpr int NT = TX * TY;
+    constexpr int NT = STEP3D_THREADS<T, TX, TY>;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ double red[32];
     __shared__ int s_last, s_it;
@@ -991,12 +1093,12 @@ step3d_batch_kernel(const BatchInst *__restrict__ insts, BatchQueue *q, int pari
     }
 }
 
-// Launch of a single-solve step kernel k (TX x TY threads, smem bytes of
+// Launch of a single-solve step kernel k (THREADS threads, smem bytes of
 // dynamic shared memory).  a.zchunk > 0: the chunked grid `grid` (tiles x
 // z-chunks).  a.zchunk <= 0: the balanced grid (PieceIter) -- as many CTAs as
 // the device holds resident at once, at most one per plane-tile.  `once`
 // and `resident` are the kernel's own per-device set-up records.
-template <int TX, int TY, typename K>
+template <int TX, int TY, int THREADS, typename K>
 cudaError_t launch_step_grid(K k, size_t smem, PerDeviceOnce &once, PerDeviceInt &resident, const StepArgs &a,
                              dim3 grid, cudaStream_t s)
 {
@@ -1004,15 +1106,15 @@ cudaError_t launch_step_grid(K k, size_t smem, PerDeviceOnce &once, PerDeviceInt
     if (a.zchunk > 0) {
         e = ensure_smem_limit(once, k, smem);
         if (e != cudaSuccess) return e;
-        k<<<grid, TX * TY, smem, s>>>(a);
+        k<<<grid, THREADS, smem, s>>>(a);
         return cudaGetLastError();
     }
     int g = 0;
-    e = persistent_grid(resident, k, smem, TX * TY, &g);
+    e = persistent_grid(resident, k, smem, THREADS, &g);
     if (e != cudaSuccess) return e;
     const long long W = (long long)a.tiles_x * ((a.n[1] + TY - 1) / TY) * a.n[2];
     if (g > W) g = static_cast<int>(W);
-    k<<<g, TX * TY, smem, s>>>(a);
+    k<<<g, THREADS, smem, s>>>(a);
     return cudaGetLastError();
 }
 

@@ -1,6 +1,5 @@
 // step3d_f64.cu -- FP64 instantiations of the fused single-solve 3D step
-// for every tile shape and
-// staging depth.
+// for every tile shape.
 #include "launchers.h"
 #include "per_device.h"
 #include "step3d.cuh"
@@ -9,39 +8,36 @@ namespace hydro {
 
 namespace {
 
-template <typename T, bool HSE, int TX, int TY, bool AS, bool GZ>
+template <typename T, bool HSE, int TX, int TY, bool GZ>
 cudaError_t launch3d_g(const StepArgs &a, dim3 grid, cudaStream_t s)
 {
-    auto k = step3d_kernel<T, HSE, TX, TY, STAGE_HANCOCK, RECON_PLM, AS, GZ>;
-    constexpr size_t smem = Step3DSmem<T, HSE, TX, TY, RECON_PLM, AS>::bytes;
+    auto k = step3d_kernel<T, HSE, TX, TY, STAGE_HANCOCK, RECON_PLM, false, GZ>;
+    constexpr size_t smem = Step3DSmem<T, HSE, TX, TY, RECON_PLM, false>::bytes;
     static PerDeviceOnce configured;   // the attribute is per function and device
     static PerDeviceInt resident;      // balanced grid size, per device
-    return launch_step_grid<TX, TY>(k, smem, configured, resident, a, grid, s);
+    return launch_step_grid<TX, TY, STEP3D_THREADS<T, TX, TY>>(k, smem, configured, resident, a, grid, s);
 }
 
 // Gravity along z only (always so with the hydrostatic background) takes the
 // kernel without the x and y gravity terms.
-template <typename T, bool HSE, int TX, int TY, bool AS>
+template <typename T, bool HSE, int TX, int TY>
 cudaError_t launch3d(const StepArgs &a, dim3 grid, cudaStream_t s)
 {
     if constexpr (HSE) {
-        return launch3d_g<T, HSE, TX, TY, AS, true>(a, grid, s);
+        return launch3d_g<T, HSE, TX, TY, true>(a, grid, s);
     } else {
-        if (a.grav[0] == 0.0 && a.grav[1] == 0.0) return launch3d_g<T, HSE, TX, TY, AS, true>(a, grid, s);
-        return launch3d_g<T, HSE, TX, TY, AS, false>(a, grid, s);
+        if (a.grav[0] == 0.0 && a.grav[1] == 0.0) return launch3d_g<T, HSE, TX, TY, true>(a, grid, s);
+        return launch3d_g<T, HSE, TX, TY, false>(a, grid, s);
     }
 }
 
 template <bool HSE>
 cudaError_t launch_v(int v, const StepArgs &a, dim3 grid, cudaStream_t s)
 {
-    switch (v) {
-    case 0: return launch3d<double, HSE, 32, 8, false>(a, grid, s);
-    case 1: return launch3d<double, HSE, 32, 4, false>(a, grid, s);
-    case 2: return launch3d<double, HSE, 16, 16, false>(a, grid, s);
-    case 4: return launch3d<double, HSE, 32, 8, true>(a, grid, s);
-    case 5: return launch3d<double, HSE, 32, 4, true>(a, grid, s);
-    case 6: return launch3d<double, HSE, 16, 16, true>(a, grid, s);
+    switch (v % 4) {   // helper warps stage in either form: one kernel per shape
+    case 0: return launch3d<double, HSE, 32, 8>(a, grid, s);
+    case 1: return launch3d<double, HSE, 32, 4>(a, grid, s);
+    case 2: return launch3d<double, HSE, 16, 16>(a, grid, s);
     default: return cudaErrorInvalidValue;
     }
 }
