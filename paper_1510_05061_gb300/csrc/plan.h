@@ -14,21 +14,22 @@ struct LaunchPlan {
     int zchunk;    // planes per CTA, or -1: the balanced grid over whole columns (PieceIter)
 };
 
-// Every candidate runs on the balanced grid (min(resident CTAs, plane-tiles)
-// CTAs with equal shares of the plane-tiles): against the z-chunks of 8 to 64
-// planes taken before, it has no partial last wave and repeats fewer planes
-// (a chunk predicts two planes and stages four beyond its own): measured on
-// GB300, us per MUSCL-Hancock step, z-chunks -> balanced, same tile: FP64 16^3
-// 288 -> 74, 101x75x130 1251 -> 1001, 128^3 1999 -> 1751; FP32 32^3 40 -> 19,
-// 128^3 147 -> 114.
+// The balanced grid (min(resident CTAs, plane-tiles) CTAs with equal shares of
+// the plane-tiles) has no partial last wave and repeats fewer planes than the
+// z-chunks of 8 to 64 planes taken before (a piece predicts two planes and
+// stages four beyond its own): measured on GB300, us per MUSCL-Hancock step, same
+// tile and kernels, FP64 16^3 288 -> 74, 101x75x130 1251 -> 1001, 128^3 1999 ->
+// 1751; FP32 32^3 40 -> 19, 128^3 147 -> 114.  Where one wave of CTAs holds every
+// tile, z-chunks of one piece per CTA can beat it, because its CTAs march parts
+// of two columns: FP64 64^3 232 against 248, 80^3 374 against 412.
 //
-// The tile is the one with the least modelled time
-//   max(alone, k unit) (ceil(W / (SMs k)) + fixed),   k = min(ctas, ceil(W / SMs)),
-// W = plane-tiles (tiles x nz), `unit` the time of a plane of one CTA divided
-// by the CTAs sharing an SM, `alone` a plane's latency on an SM of its own,
-// `fixed` the planes' worth of work a CTA repeats; the constants are fitted to
-// the same sweep (16^3 .. 320^3, 200x40x100, 300x40x200) and reproduce its
-// times within 10 %.
+// Tile and partition are those with the least modelled time, with
+//   time = max(alone, k unit) (planes + pieces fixed),   k = min(ctas, ceil(W / SMs)),
+// planes and pieces of the longest CTA, W = plane-tiles (tiles x nz), `unit` the
+// time of a plane of one CTA divided by the CTAs sharing an SM, `alone` a
+// plane's latency on an SM of its own, `fixed` the planes' worth of work a piece
+// repeats.  The constants are fitted to sweeps from 16^3 to 320^3, 200x40x100 and
+// 300x40x200 and reproduce their times within 10 %.
 struct TileCost {
     int variant, ctas;
     double alone, unit, fixed;   // us
@@ -38,16 +39,17 @@ inline LaunchPlan default_plan(const hydro_problem &p)
 {
     constexpr int SMS = 152;
     const bool fp32 = p.precision == HYDRO_FP32;
-    // FP64: 16 x 16 tiles, 32 x 8 where they fit the grid better (200x40x100:
-    // 838 against 875 us), 32 x 4 for grids of few tiles (16^3: 61 against 74 us)
-    static const TileCost f64[] = {{6, 1, 31.0, 31.0, 2.45}, {4, 1, 33.2, 33.2, 2.3}, {5, 1, 25.6, 25.6, 1.4}};
+    // FP64: 16 x 16 tiles (128^3: 1356 us, 32 x 8 1593, 32 x 4 2141), 32 x 8 where
+    // those waste more of the grid, 32 x 4 for grids of few tiles (16^3: 50
+    // against 70 us)
+    static const TileCost f64[] = {{2, 1, 24.0, 24.0, 1.2}, {0, 1, 28.2, 28.2, 1.2}, {1, 1, 19.5, 19.5, 1.2}};
     // FP32: 32 x 8 tiles, three CTAs per SM; 32 x 16, one CTA; 16 x 16, two;
     // 32 x 4 for the smallest grids
-    static const TileCost f32[] = {{0, 3, 3.5, 1.86, 2.3}, {3, 1, 3.76, 3.76, 2.3}, {2, 2, 3.5, 2.1, 2.3},
-                                   {5, 4, 3.0, 1.2, 2.3}};
+    static const TileCost f32[] = {{0, 3, 3.5, 1.86, 1.2}, {3, 1, 3.76, 3.76, 1.2}, {2, 2, 3.5, 2.1, 1.2},
+                                   {5, 4, 3.0, 1.2, 1.2}};
     // piecewise parabolic stages hold two more planes and a deeper halo: the
     // 512-thread tile is the fastest by a quarter (128^3: 327 against 422 us)
-    static const TileCost f32_ppm[] = {{3, 1, 3.76, 3.76, 3.5}};
+    static const TileCost f32_ppm[] = {{3, 1, 3.76, 3.76, 1.8}};
     const TileCost *c = fp32 ? (p.recon == HYDRO_RECON_PPM ? f32_ppm : f32) : f64;
     const int nc = fp32 ? (p.recon == HYDRO_RECON_PPM ? 1 : 4) : 3;
     LaunchPlan best{c[0].variant, -1};
@@ -57,10 +59,24 @@ inline LaunchPlan default_plan(const hydro_problem &p)
         const long long W = (long long)((p.n[0] + s.tx - 1) / s.tx) * ((p.n[1] + s.ty - 1) / s.ty) * p.n[2];
         const long long k = std::min<long long>(c[i].ctas, (W + SMS - 1) / SMS);
         const long long planes = (W + SMS * k - 1) / (SMS * k);
-        const double t = std::max(c[i].alone, k * c[i].unit) * (planes + c[i].fixed);
+        const long long tiles = W / p.n[2], G = SMS * k;
+        const double tp = std::max(c[i].alone, k * c[i].unit);
+        // the balanced grid's longest CTA, which marches parts of two columns
+        // unless the shares divide the columns; or, where one wave holds every
+        // tile, z-chunks of one piece each
+        const bool split = planes > 1 && !(G % tiles == 0 && p.n[2] % (G / tiles) == 0);
+        double t = tp * (planes + (split ? 2 : 1) * c[i].fixed);
+        int z = -1;
+        if (tiles <= G) {
+            const int zc = (int)((p.n[2] + G / tiles - 1) / (G / tiles));
+            if (tp * (zc + c[i].fixed) < t) {
+                t = tp * (zc + c[i].fixed);
+                z = zc;
+            }
+        }
         if (i == 0 || t < tbest) {
             tbest = t;
-            best.variant = c[i].variant;
+            best = LaunchPlan{c[i].variant, z};
         }
     }
     // an FP32 state well beyond the 129 MB L2: 32 x 8 tiles on z-chunks of 32
