@@ -15,8 +15,7 @@ static cudaError_t launch_ctu(const StepArgs &a, dim3 grid, cudaStream_t s)
     static PerDeviceOnce configured;   // the attribute is per function and device
     const cudaError_t e = ensure_smem_limit(configured, k, smem);
     if (e != cudaSuccess) return e;
-    k<<<grid, TX * TY, smem, s>>>(a);
-    return cudaGetLastError();
+    return launch_step<true>(k, grid, TX * TY, smem, s, a);
 }
 
 cudaError_t launch_ctu2d(const StepArgs &a, dim3 grid, cudaStream_t s, bool fp32)

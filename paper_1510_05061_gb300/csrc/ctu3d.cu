@@ -43,13 +43,12 @@ cudaError_t launch_ctu(const StepArgs &a0, cudaStream_t s)
         // marched at the same heights keep their halo rows in L2
         a.zchunk = 0;
         const long long W = (long long)a.tiles_x * ((a.n[1] + TY - 1) / TY) * a.n[2];
-        k<<<(int)std::min<long long>(g, W), NT, smem, s>>>(a);
+        return launch_step<false>(k, (int)std::min<long long>(g, W), NT, smem, s, a);
     } else {
         a.zchunk = ctu_zchunk(a.n, sizeof(T) == 4);
         const dim3 grid(a.tiles_x * ((a.n[1] + TY - 1) / TY), (a.n[2] + a.zchunk - 1) / a.zchunk);
-        k<<<grid, NT, smem, s>>>(a);
+        return launch_step<true>(k, grid, NT, smem, s, a);
     }
-    return cudaGetLastError();
 }
 
 }  // namespace

@@ -754,6 +754,16 @@ __device__ __forceinline__ double block_max_t(T v, double *red)
     return double(v);
 }
 
+// First act of a step kernel (launch_step): waits for the kernel before
+// it in the stream to end, its writes visible, then lets the next one's CTAs
+// take SMs as this kernel's leave them.  Nothing of the previous step is read
+// before the wait.  Without a chained launch both are no-ops.
+__device__ __forceinline__ void chain_begin()
+{
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
 // Last-CTA finalisation of a step's time control.  Each of the nblocks
 // contributions (CTAs, or work items of one instance) calls it once with its
 // max signal speed (valid in thread 0), whether any of its cells failed the

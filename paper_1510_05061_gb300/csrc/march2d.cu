@@ -23,8 +23,7 @@ cudaError_t launch_nt(const StepArgs &a0, cudaStream_t s)
     a.tiles_x = (a.n[0] + March2DSmem<T, NT>::UX - 1) / March2DSmem<T, NT>::UX;
     const long long rows = (long long)a.tiles_x * a.n[1];
     g = (int)std::min<long long>(std::min(g, MARCH2D_MAX_CTAS), rows);
-    k<<<g, NT, smem, s>>>(a);
-    return cudaGetLastError();
+    return launch_step<true>(k, g, NT, smem, s, a);
 }
 
 template <int ST>

@@ -267,6 +267,7 @@ __global__ void __launch_bounds__(NT, (sizeof(T) == 4 ? 768 : 384) / NT) march2d
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ double red[32];
     __shared__ int s_last;
+    chain_begin();
     const double t_now = a.ctrl->t;
     const double dt_cfl = a.ctrl->dt_next;
     // frozen: nothing moves (the host finds the current buffer from the step count)

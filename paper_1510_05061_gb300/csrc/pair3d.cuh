@@ -521,6 +521,7 @@ __global__ void __launch_bounds__(TXP * TY, MINB) step3d_pair_kernel(const StepA
     __shared__ double red[32];
     __shared__ int s_last;
     const int tile = blockIdx.x, chunk = blockIdx.y;
+    chain_begin();
     const double t_now = a.ctrl->t;
     const double dt_cfl = a.ctrl->dt_next;
     // frozen: nothing moves (the host finds the current buffer from the step count)

@@ -17,8 +17,7 @@ cudaError_t launch_pair(const StepArgs &a, dim3 grid, cudaStream_t s)
     static PerDeviceOnce configured;   // the attribute is per function and device
     const cudaError_t e = ensure_smem_limit(configured, k, smem);
     if (e != cudaSuccess) return e;
-    k<<<grid, TXP * TY, smem, s>>>(a);
-    return cudaGetLastError();
+    return launch_step<true>(k, grid, TXP * TY, smem, s, a);
 }
 
 template <bool HSE, int TXP, int TY, int MINB>

@@ -16,7 +16,7 @@ cudaError_t launch3d(const StepArgs &a, dim3 grid, cudaStream_t s)
     constexpr size_t smem = Step3DSmem<double, HSE, TX, TY, RC>::bytes;
     static PerDeviceOnce configured;   // the attribute is per function and device
     static PerDeviceInt resident;      // balanced grid size, per device
-    return launch_step_grid<TX, TY, STEP3D_THREADS<double, TX, TY>>(k, smem, configured, resident, a, grid, s);
+    return launch_step_grid<TX, TY, STEP3D_THREADS<double, TX, TY>, false>(k, smem, configured, resident, a, grid, s);
 }
 
 template <int ST, int RC, bool HSE>

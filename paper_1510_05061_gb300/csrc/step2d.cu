@@ -19,8 +19,7 @@ cudaError_t launch2d(const StepArgs &a0, cudaStream_t s)
     if (e != cudaSuccess) return e;
     StepArgs a = a0;
     a.tiles_x = (a.n[0] + TX - 1) / TX;
-    k<<<a.tiles_x * ((a.n[1] + TY - 1) / TY), TX * TY, smem, s>>>(a);
-    return cudaGetLastError();
+    return launch_step<true>(k, a.tiles_x * ((a.n[1] + TY - 1) / TY), TX * TY, smem, s, a);
 }
 
 template <int ST, int RC>

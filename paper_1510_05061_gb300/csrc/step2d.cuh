@@ -325,6 +325,7 @@ __global__ void __launch_bounds__(TX * TY, sizeof(T) == 8 ? 768 / (TX * TY) : 1)
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ double red[32];
     __shared__ int s_last;
+    chain_begin();
     const double t_now = a.ctrl->t;
     const double dt_cfl = a.ctrl->dt_next;
     // frozen: nothing moves (the host finds the current buffer from the step count)

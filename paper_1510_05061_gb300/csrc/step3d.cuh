@@ -421,7 +421,8 @@ __device__ __forceinline__ void step3d_body(const StepArgs &a, int tile, int z0,
     };
 
     // the planes before the march (with helpers: by every thread of the CTA, a
-    // few elements of different planes in flight each)
+    // few elements of different planes in flight each; the FP32 kernels lose 2 to
+    // 8 % with it to another register allocation)
     auto stage_first = [&](int pz0) {
         constexpr int NP = H + LEAD - 1, NA = NT + STEP3D_HELPERS<T>, NE = (NP * HXY + NA - 1) / NA;
 #pragma unroll
@@ -1016,6 +1017,7 @@ step3d_kernel(const StepArgs a)
     // time control: dt from the device block, clamped to t_end (both
     // Runge-Kutta stages read the same block: the first stage leaves it
     // unchanged apart from its error bits)
+    chain_begin();
     const double t_now = a.ctrl->t;
     const double dt_cfl = a.ctrl->dt_next;
     // frozen (time at t_end, step limit reached, or error state): nothing
@@ -1098,7 +1100,7 @@ step3d_batch_kernel(const BatchInst *__restrict__ insts, BatchQueue *q, int pari
 // z-chunks).  a.zchunk <= 0: the balanced grid (PieceIter) -- as many CTAs as
 // the device holds resident at once, at most one per plane-tile.  `once`
 // and `resident` are the kernel's own per-device set-up records.
-template <int TX, int TY, int THREADS, typename K>
+template <int TX, int TY, int THREADS, bool CHAIN, typename K>
 cudaError_t launch_step_grid(K k, size_t smem, PerDeviceOnce &once, PerDeviceInt &resident, const StepArgs &a,
                              dim3 grid, cudaStream_t s)
 {
@@ -1106,16 +1108,14 @@ cudaError_t launch_step_grid(K k, size_t smem, PerDeviceOnce &once, PerDeviceInt
     if (a.zchunk > 0) {
         e = ensure_smem_limit(once, k, smem);
         if (e != cudaSuccess) return e;
-        k<<<grid, THREADS, smem, s>>>(a);
-        return cudaGetLastError();
+        return launch_step<CHAIN>(k, grid, THREADS, smem, s, a);
     }
     int g = 0;
     e = persistent_grid(resident, k, smem, THREADS, &g);
     if (e != cudaSuccess) return e;
     const long long W = (long long)a.tiles_x * ((a.n[1] + TY - 1) / TY) * a.n[2];
     if (g > W) g = static_cast<int>(W);
-    k<<<g, THREADS, smem, s>>>(a);
-    return cudaGetLastError();
+    return launch_step<CHAIN>(k, g, THREADS, smem, s, a);
 }
 
 }  // namespace hydro

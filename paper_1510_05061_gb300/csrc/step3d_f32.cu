@@ -16,7 +16,7 @@ cudaError_t launch3d(const StepArgs &a, dim3 grid, cudaStream_t s)
     constexpr size_t smem = Step3DSmem<T, HSE, TX, TY, RECON_PLM, AS>::bytes;
     static PerDeviceOnce configured;   // the attribute is per function and device
     static PerDeviceInt resident;      // balanced grid size, per device
-    return launch_step_grid<TX, TY, STEP3D_THREADS<T, TX, TY>>(k, smem, configured, resident, a, grid, s);
+    return launch_step_grid<TX, TY, STEP3D_THREADS<T, TX, TY>, true>(k, smem, configured, resident, a, grid, s);
 }
 
 template <bool HSE>

@@ -15,7 +15,7 @@ cudaError_t launch3d_g(const StepArgs &a, dim3 grid, cudaStream_t s)
     constexpr size_t smem = Step3DSmem<T, HSE, TX, TY, RECON_PLM, false>::bytes;
     static PerDeviceOnce configured;   // the attribute is per function and device
     static PerDeviceInt resident;      // balanced grid size, per device
-    return launch_step_grid<TX, TY, STEP3D_THREADS<T, TX, TY>>(k, smem, configured, resident, a, grid, s);
+    return launch_step_grid<TX, TY, STEP3D_THREADS<T, TX, TY>, false>(k, smem, configured, resident, a, grid, s);
 }
 
 // Gravity along z only (always so with the hydrostatic background) takes the
