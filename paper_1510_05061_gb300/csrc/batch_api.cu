@@ -19,6 +19,7 @@
 #include <vector>
 
 #include "../../include/hydro.h"
+#include "batch_plan.h"
 #include "host_pages.h"
 #include "hydro_internal.h"
 #include "launchers.h"
@@ -146,6 +147,7 @@ struct hydro_batch {
     cudaStream_t stream;
     int parity;                // parity of the next launch
     int variant, zchunk;       // zchunk: longest chunk of an instance's column (0 = default)
+    bool even, pick;           // columns in equal shares (batch_plan), and the variant of its choice
     bool dirty;                // queue / tables need an upload
     bool use_graph;
     BatchQueue *d_queue;
@@ -228,10 +230,19 @@ int ensure_pinned(hydro_batch *b, int k, size_t need)
 // kernels or grids change, not when the membership does.
 int rebuild(hydro_batch *b)
 {
+    BatchPlan plan{};
+    if (b->even) {
+        std::vector<const hydro_problem *> p3;
+        for (const InstInfo &I : b->inst)
+            if (I.active && I.prob.ndim == 3) p3.push_back(&I.prob);
+        if (!p3.empty()) plan = batch_plan(p3.data(), (int)p3.size(), b->precision == HYDRO_FP32, b->pick ? -1 : b->variant);
+        if (plan.shares > 0) b->variant = plan.variant;
+    }
     const TileShape ts = TILE3D_SHAPES[b->variant];
     std::vector<BatchInst> insts(b->max_instances, BatchInst{});
     std::vector<BatchItem> items3, items2;
     std::vector<int> len3;
+    CutState cut{};
     for (int i = 0; i < (int)b->inst.size(); ++i) {
         const InstInfo &I = b->inst[i];
         if (!I.active) continue;
@@ -272,23 +283,32 @@ int rebuild(hydro_batch *b)
             fill_fp32_constants(a);
         }
         int local = 0;
+        if (is3 && plan.shares > 0) {
+            cut_columns(plan, i, tiles_x * tiles_y, p.n[2], cut, items3, &local);
+            bi.nitems = local;
+            continue;
+        }
         for (int c = 0; c < nch; ++c)
             for (int t = 0; t < tiles_x * tiles_y; ++t) {
                 if (is3) {
-                    items3.push_back(BatchItem{i, t, c, local++});
-                    len3.push_back(std::min(zc, p.n[2] - c * zc));
+                    items3.push_back(BatchItem{i, t, c * zc, std::min((c + 1) * zc, p.n[2]), local++, -1});
+                    len3.push_back(items3.back().z1 - items3.back().z0);
                 } else {
-                    items2.push_back(BatchItem{i, t, c, local++});
+                    items2.push_back(BatchItem{i, t, 0, 0, local++, -1});
                 }
             }
     }
     if ((long long)items3.size() > b->cap3 || (long long)items2.size() > b->cap2) return HYDRO_ERR_OOM;
-    // largest first (stable: an instance's items stay in tile order)
-    std::vector<int> order(items3.size());
-    for (size_t k = 0; k < order.size(); ++k) order[k] = (int)k;
-    std::stable_sort(order.begin(), order.end(), [&](int x, int y) { return len3[x] > len3[y]; });
-    std::vector<BatchItem> sorted3(items3.size());
-    for (size_t k = 0; k < order.size(); ++k) sorted3[k] = items3[order[k]];
+    std::vector<BatchItem> sorted3;
+    if (plan.shares > 0) {
+        sorted3 = claim_order(items3);
+    } else {
+        // largest first (stable: an instance's items stay in tile order)
+        std::vector<int> order(items3.size());
+        for (size_t k = 0; k < order.size(); ++k) order[k] = (int)k;
+        std::stable_sort(order.begin(), order.end(), [&](int x, int y) { return len3[x] > len3[y]; });
+        for (int k : order) sorted3.push_back(items3[k]);
+    }
 
     b->nitems3 = (int)sorted3.size();
     b->nitems2 = (int)items2.size();
@@ -307,7 +327,7 @@ int rebuild(hydro_batch *b)
     BatchQueue qh{};
     qh.items[0] = b->d_items3;
     qh.items[1] = b->d_items2;
-    qh.nitems[0] = b->nitems3;
+    qh.nitems[0] = plan.shares > 0 ? cut.shares : b->nitems3;
     qh.nitems[1] = b->nitems2;
     std::memcpy(pin + o_q, &qh, q_bytes);
     cudaError_t e = cudaMemcpyAsync(b->d_insts, pin, bi_bytes, cudaMemcpyHostToDevice, b->stream);
@@ -657,7 +677,9 @@ int hydro_batch_init(const hydro_problem *probs, int count, void *const *Ua, voi
         if (rc) break;
         w += inst_layout(probs[i]).total;
     }
+    b->even = b->pick = true;
     if (rc == HYDRO_OK) rc = rebuild(b);
+    b->pick = false;   // later changes of membership keep the kernel
     if (rc) {
         hydro_batch_destroy(b);
         return rc;
@@ -671,6 +693,7 @@ int hydro_batch_configure(hydro_batch *b, int variant, int zchunk)
     if (!b || !tile3d_available(variant, b->precision == HYDRO_FP32) || zchunk < 0) return HYDRO_ERR_INVALID_ARG;
     b->variant = variant;
     b->zchunk = zchunk;
+    b->even = false;
     return rebuild(b);
 }
 

@@ -817,9 +817,11 @@ __device__ __forceinline__ void finish_step(double smax_cta, bool bad_cta, const
 // exhausted.  The CTA that is last to find the list exhausted resets the
 // counters (every other CTA has stopped claiming by then), so the next
 // launch of this parity starts from item 0.  Every thread must call it.
-__device__ __forceinline__ int claim_item(BatchQueue *q, int L, int parity, int *s_it)
+__device__ __forceinline__ int claim_item(BatchQueue *q, int L, int parity, int *s_it, int next = -1)
 {
-    if (threadIdx.x == 0) {
+    if (threadIdx.x == 0 && next >= 0) {
+        *s_it = next;
+    } else if (threadIdx.x == 0) {
         const int n = q->nitems[L];
         int it = (int)atomicAdd(&q->next[L][parity], 1u);
         if (it >= n) {

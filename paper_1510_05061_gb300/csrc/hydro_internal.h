@@ -82,12 +82,14 @@ inline void fill_fp32_constants(StepArgs &a)
     }
 }
 
-// One item of a batched step's work list: a tile and z-chunk of one instance.
+// One item of a batched step's work list: a piece of a tile's column of one
+// instance (2D: the tile).
 struct BatchItem {
     int inst;    // instance index
     int tile;    // tile within the instance's x-y tiling
-    int chunk;   // z-chunk (0 in 2D)
+    int z0, z1;  // planes (unused in 2D)
     int local;   // index of this item among the instance's items (its partial slot)
+    int next;    // index of the item to take after this one without a claim, or -1
 };
 
 // Per-instance launch arguments for both ping-pong parities.
@@ -107,7 +109,7 @@ struct BatchInst {
 // out of items resets the counter and the exit count for the next launch.
 struct BatchQueue {
     const BatchItem *items[2];   // [0]: 3D items, [1]: 2D items
-    int nitems[2];
+    int nitems[2];               // items to claim (the first of the list; the others follow by `next`)
     unsigned next[2][2];         // [list][parity]: next unclaimed item
     unsigned exited[2][2];       // [list][parity]: CTAs that found no item left
 };

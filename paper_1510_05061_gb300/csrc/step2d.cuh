@@ -345,8 +345,8 @@ __global__ void __launch_bounds__(TX * TY, sizeof(T) == 8 ? 768 / (TX * TY) : 1)
 }
 
 // Persistent batched 2D step over the queue's 2D list of (instance, tile)
-// items; the BatchItem/BatchInst layout is shared with the 3D batch (chunk
-// unused).  Frozen instances are skipped.
+// items; the BatchItem/BatchInst layout is shared with the 3D batch (z0,
+// z1 and next unused).  Frozen instances are skipped.
 template <typename T, int TX, int TY>
 __global__ void __launch_bounds__(TX * TY)
 step2d_batch_kernel(const BatchInst *__restrict__ insts, BatchQueue *q, int parity)

@@ -1067,14 +1067,17 @@ step3d_batch_kernel(const BatchInst *__restrict__ insts, BatchQueue *q, int pari
     __shared__ double red[32];
     __shared__ int s_last, s_it;
     __shared__ StepArgs sa;
+    __shared__ BatchItem s_w;   // (per-thread copies held registers through the march: 2.9 % slower)
     const BatchItem *items = q->items[0];
+    int next = -1;
     for (;;) {
-        const int it = claim_item(q, 0, parity, &s_it);
+        const int it = claim_item(q, 0, parity, &s_it, next);
         if (it < 0) break;
-        const BatchItem w = items[it];
+        const int inst = items[it].inst;
+        if (threadIdx.x == 0) { s_w = items[it]; next = s_w.next; }
         if (threadIdx.x < (int)(sizeof(StepArgs) / sizeof(int))) {
             reinterpret_cast<int *>(&sa)[threadIdx.x] =
-                reinterpret_cast<const int *>(&insts[w.inst].a[parity])[threadIdx.x];
+                reinterpret_cast<const int *>(&insts[inst].a[parity])[threadIdx.x];
         }
         __syncthreads();
         const double t_now = sa.ctrl->t;
@@ -1083,13 +1086,10 @@ step3d_batch_kernel(const BatchInst *__restrict__ insts, BatchQueue *q, int pari
             const double dtd = (dt_cfl >= sa.t_end - t_now) ? sa.t_end - t_now : dt_cfl;
             T smax;
             bool bad;
-            const int z0 = w.chunk * sa.zchunk;
-            step3d_body<T, HSE, TX, TY, STAGE_HANCOCK, RECON_PLM, AS>(sa, w.tile, z0, min(z0 + sa.zchunk, sa.n[2]),
-                                                                      dtd, smem_raw, smax,
-                                                                      bad);
+            step3d_body<T, HSE, TX, TY, STAGE_HANCOCK, RECON_PLM, AS>(sa, s_w.tile, s_w.z0, s_w.z1, dtd, smem_raw, smax, bad);
             const bool bad_cta = __syncthreads_or(bad) != 0;
             const double m = block_max_t<NT, T>(smax, red);
-            finish_step<NT>(m, bad_cta, sa, insts[w.inst].nitems, w.local, dtd, true, &s_last);
+            finish_step<NT>(m, bad_cta, sa, insts[s_w.inst].nitems, s_w.local, dtd, true, &s_last);
         }
         __syncthreads();
     }
