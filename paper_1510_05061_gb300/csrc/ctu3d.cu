@@ -1,7 +1,6 @@
 // ctu3d.cu -- FP64 and FP32 instantiations of the fused 3D corner transport
-// upwind step.  Tiles: FP32 16 x 16 (256 threads, 152 KB of shared memory),
-// FP64 16 x 8 (256 threads, 171 KB); FP32 z-chunks sized for several waves
-// of the 152 SMs (one CTA per SM), FP64 the balanced grid.
+// upwind step.  Tiles: FP32 16 x 16 (512 threads, 152 KB of shared memory),
+// FP64 16 x 8 (256 threads, 171 KB); one CTA per SM.
 #include <algorithm>
 
 #include "ctu3d.cuh"
@@ -15,13 +14,19 @@ namespace {
 constexpr int CTU_TX = 16;
 int ctu_ty(bool fp32) { return fp32 ? 16 : 8; }
 
-// planes per CTA: at least 8 waves of one CTA per SM, chunks of 8 or more
-int ctu_zchunk(const int n[3], bool fp32)
+// z partition of T tiles of nz planes on G resident CTAs, one per SM: 0, the
+// balanced grid (equal shares of the plane-tiles, no partial last wave), or the
+// planes of z-chunks, one piece per CTA, where they cost less: a piece predicts
+// two planes beside its own, and a balanced CTA marches parts of two columns.  us
+// per step, chunks of 8 planes and more in several waves -> balanced / one
+// piece, FP32: 16^3 44 -> 18 / 17, 80^3 89 -> 78 / 73, 101x75x130 189 -> 148 /
+// 152, 128^3 318 -> 253 / 292, 240^3 1702 -> 1627; FP64 balanced / one piece:
+// 40^3 225 / 182, 80^3 969 / 921, 64^3 548 / 568, 128^3 3605 / 4202.
+int ctu_partition(long long T, int nz, int G)
 {
-    const long long tiles = (long long)((n[0] + CTU_TX - 1) / CTU_TX) * ((n[1] + ctu_ty(fp32) - 1) / ctu_ty(fp32));
-    long long nch = (8ll * 152 + tiles - 1) / tiles;
-    nch = std::min(nch, std::max(1ll, (long long)(n[2] / 8)));
-    return (int)((n[2] + nch - 1) / nch);
+    if (T > G) return 0;
+    const int zc = (int)((nz + G / T - 1) / (G / T));
+    return zc + 2.0 <= std::max(1.0, (double)T * nz / G) + 4.0 ? zc : 0;
 }
 
 template <typename T, bool HSE, int TX, int TY, bool GZ>
@@ -36,19 +41,11 @@ cudaError_t launch_ctu(const StepArgs &a0, cudaStream_t s)
     if (e != cudaSuccess) return e;
     StepArgs a = a0;
     a.tiles_x = (a.n[0] + TX - 1) / TX;
-    if constexpr (sizeof(T) == 8) {
-        // FP64: the balanced grid, every resident CTA marching an equal share
-        // of the plane-tiles (no partial last wave; measured +8 % at RT 256^3).
-        // FP32 keeps z-chunks: the same speed there, and neighbouring tiles
-        // marched at the same heights keep their halo rows in L2
-        a.zchunk = 0;
-        const long long W = (long long)a.tiles_x * ((a.n[1] + TY - 1) / TY) * a.n[2];
-        return launch_step<false>(k, (int)std::min<long long>(g, W), NT, smem, s, a);
-    } else {
-        a.zchunk = ctu_zchunk(a.n, sizeof(T) == 4);
-        const dim3 grid(a.tiles_x * ((a.n[1] + TY - 1) / TY), (a.n[2] + a.zchunk - 1) / a.zchunk);
-        return launch_step<true>(k, grid, NT, smem, s, a);
-    }
+    const long long tiles = (long long)a.tiles_x * ((a.n[1] + TY - 1) / TY);
+    a.zchunk = ctu_partition(tiles, a.n[2], g);
+    const dim3 grid = a.zchunk > 0 ? dim3((unsigned)tiles, (a.n[2] + a.zchunk - 1) / a.zchunk)
+                                   : dim3((unsigned)std::min<long long>(g, tiles * a.n[2]));
+    return launch_step<sizeof(T) == 4>(k, grid, NT, smem, s, a);
 }
 
 }  // namespace

@@ -152,13 +152,25 @@ __device__ __forceinline__ void predict_axis_f64(const double (&w)[5], const dou
     if (HSE && d == 2) wd[3] = fma_rn(-mul_rn(hdt, bg.B), rinv, wd[3]);
 }
 
-// FP64 runs 256 threads on its 16 x 8 tile (two warps for each of the SM's
-// four FP64 units instead of one): the loops over ring cells, faces and
-// corrections stride by the CTA's threads, not by the tile's cells, and the
-// faces and the corrections of all three axes form one list each (the axis a
-// run-time value), so that their last, partial warps do not add up.
+// Twice the tile's cells in threads: the loops over ring cells, faces and
+// corrections stride by the CTA's threads, not by the tile's cells.  FP64: two
+// warps for each of the SM's four FP64 units instead of one on its 16 x 8
+// tile, and the faces and the corrections of all three axes form one list each (the
+// axis a run-time value), so that their last, partial warps do not add up.
+// FP32: 16 instead of 8 warps on the one 16 x 16 CTA that shared memory holds,
+// and one pass over each axis's 306 to 324 faces instead of two, the axes'
+// lists begun on different warps (ctu_first) so that no warp runs all three.
+// Same z-chunks, 256 threads -> 512: 128^3 421 -> 318 us, 32^3 60 -> 46, 240^3
+// 2302 -> 1702; the lists' first threads: 128^3 253 -> 246, 240^3 1627 -> 1576.
 template <typename T, int TX, int TY>
-constexpr int CTU3D_THREADS = sizeof(T) == 8 ? 256 : TX * TY;
+constexpr int CTU3D_THREADS = 2 * TX * TY;
+
+// First item of a loop over a list whose item 0 falls on thread `from`.
+template <int NT>
+__device__ __forceinline__ int ctu_first(int tid, int from)
+{
+    return (tid + NT - from) % NT;
+}
 
 template <typename T, bool HSE, int TX, int TY, bool GZ>
 __device__ __forceinline__ void ctu3d_body(const StepArgs &a, int tile, int z0, int z1, double dtd,
@@ -184,7 +196,7 @@ __device__ __forceinline__ void ctu3d_body(const StepArgs &a, int tile, int z0, 
     const long long vs = a.vstride;
     const int plane = static_cast<int>(a.plane);
     const int gx = x0 + tx, gy = y0 + ty;
-    const bool cell = NT == TX * TY || tid < TX * TY;   // the thread has a cell of the tile
+    const bool cell = tid < TX * TY;   // the thread has a cell of the tile
     const bool own = cell && gx < nx && gy < ny;
     const int own_off = gy * nx + gx;
     const T dt = T(dtd), hdt = T(0.5) * T(dtd);
@@ -536,7 +548,7 @@ __device__ __forceinline__ void ctu3d_body(const StepArgs &a, int tile, int z0, 
 #pragma unroll
                 for (int q = 0; q < NV; ++q) FX(b, q, cy, fi) = f[q];
             }
-            for (int i = rotated_start<NT>(tid); i < EX * (TY + 1); i += NT) {   // second pass off warp 0
+            for (int i = ctu_first<NT>(tid, 320); i < EX * (TY + 1); i += NT) {
                 const int cx = i % EX - 1, fj = i / EX;
                 T f[NV];
                 y_face(b, p, fj, cx, f);
@@ -544,7 +556,7 @@ __device__ __forceinline__ void ctu3d_body(const StepArgs &a, int tile, int z0, 
                 for (int q = 0; q < NV; ++q) FY(b, q, fj, cx) = f[q];
             }
             if (p >= z0) {
-                for (int i = tid; i < EX * EY; i += NT) {
+                for (int i = ctu_first<NT>(tid, 128); i < EX * EY; i += NT) {
                     const int cx = i % EX - 1, cy = i / EX - 1;
                     T f[NV];
                     z_face(p, 5, cy, cx, f);
@@ -587,7 +599,7 @@ __device__ __forceinline__ void ctu3d_body(const StepArgs &a, int tile, int z0, 
                 correct(b, 4, 4, 6, cy, cx, dx1, hdt_dx[0], dy1, hdt_dx[1], rbz, pbz, T(0));
             }
             if (out_plane) {
-                for (int i = tid; i < EX * TY; i += NT) {        // x states: columns -1..TX, tile rows
+                for (int i = ctu_first<NT>(tid, 256); i < EX * TY; i += NT) {   // x states: columns -1..TX, tile rows
                     const int cx = i % EX - 1, cy = i / EX;
                     T dy1[NV], dz1[NV];
 #pragma unroll
@@ -597,8 +609,8 @@ __device__ __forceinline__ void ctu3d_body(const StepArgs &a, int tile, int z0, 
                     }
                     correct(bm, 0, 0, 1, cy, cx, dy1, hdt_dx[1], dz1, hdt_dx[2], rbc, pbc, dmz);
                 }
-                // y states: tile columns, rows -1..TY (second pass off warp 0)
-                for (int i = rotated_start<NT>(tid); i < TX * EY; i += NT) {
+                // y states: tile columns, rows -1..TY
+                for (int i = ctu_first<NT>(tid, 32); i < TX * EY; i += NT) {
                     const int cx = i % TX, cy = i / TX - 1;
                     T dx1[NV], dz1[NV];
 #pragma unroll
@@ -618,19 +630,19 @@ __device__ __forceinline__ void ctu3d_body(const StepArgs &a, int tile, int z0, 
             // x and y faces from the warps without a cell on
             constexpr int NFX = (TX + 1) * TY, NFY = TX * (TY + 1);
             if (out_plane)
-                for (int i = (tid + NT - TX * TY) % NT; i < NFX + NFY; i += NT) {
+                for (int i = ctu_first<NT>(tid, TX * TY); i < NFX + NFY; i += NT) {
                     const int ax = i < NFX ? 0 : 1, j = i - (ax ? NFX : 0), w = ax ? TX : TX + 1;
                     any_face(ax, p - 1, bm, bm, 6, j % w, j / w);
                 }
         } else if (out_plane) {
-            for (int i = tid; i < (TX + 1) * TY; i += NT) {
+            for (int i = ctu_first<NT>(tid, 256); i < (TX + 1) * TY; i += NT) {
                 const int fi = i % (TX + 1), cy = i / (TX + 1);
                 T f[NV];
                 x_face(bm, p - 1, cy, fi, f);
 #pragma unroll
                 for (int q = 0; q < NV; ++q) FX(bm, q, cy, fi) = f[q];
             }
-            for (int i = rotated_start<NT>(tid); i < TX * (TY + 1); i += NT) {
+            for (int i = ctu_first<NT>(tid, 32); i < TX * (TY + 1); i += NT) {
                 const int cx = i % TX, fj = i / TX;
                 T f[NV];
                 y_face(bm, p - 1, fj, cx, f);
