@@ -267,13 +267,14 @@ __device__ __forceinline__ T signal_speed(const T *m, T rinv, T c, const T (&inv
     return fma(rinv, a, c * sidx);
 }
 
-// A double cut to FP32 on the integer pipe (a conversion instruction holds
-// the FP64 pipe like a multiply): relative error below 2^-22; 0 below FP32's
-// normal range, infinity beyond it.
-__device__ __forceinline__ float cut_f32(double x)
+// A double divided by 2^k and cut to FP32 on the integer pipe (a conversion
+// instruction holds the FP64 pipe like a multiply), bias = 0x38000000 + (k << 20)
+// between 0x00100000 and 0x70000000: relative error below 2^-22; 0 below FP32's
+// normal range, infinity beyond it and for infinities and NaN.
+__device__ __forceinline__ float cut_f32(double x, int bias)
 {
     const unsigned hi = __double2hiint(x), lo = __double2loint(x);
-    const unsigned v = (hi & 0x7fffffffu) - 0x38000000u;   // exponent rebiased, three bits above FP32's place
+    const unsigned v = (hi & 0x7fffffffu) - static_cast<unsigned>(bias);   // exponent rebiased, three bits above FP32's place
     unsigned f = __funnelshift_l(lo, v, 3);
     f = static_cast<int>(v) < 0x00100000 ? 0u : (v >= 0x0ff00000u ? 0x7f800000u : f);
     return __uint_as_float(f | (hi & 0x80000000u));
@@ -281,21 +282,35 @@ __device__ __forceinline__ float cut_f32(double x)
 
 // Whether an FP64 cell's new state u (background rb, pb) is certainly
 // admissible and its CFL signal speed certainly below `below` (or just
-// finite, for below = infinity): an FP32 estimate whose margins, 1e-5 of every
-// term, cover its 2^-22 conversions and rounded operations many times over.
-// The grid's maximum is exact, so a cell below a speed some cell has reached
-// needs no FP64 evaluation; false only means that it has to be evaluated.
+// finite, for below = infinity), from an FP32 estimate.  The grid's maximum is
+// exact, so a cell below a speed some cell has reached needs no FP64
+// evaluation; false only means that it has to be evaluated.
+//
+// The state is divided by a power of two near the cell's density (HSE: the
+// background's), which changes neither velocities nor the sound speed: with r
+// from 1/4 to 1e30 nothing depends on the unit of mass, and where the units of
+// length and time put an intermediate near the ends of FP32's range the answer
+// is false.  What is lost below:
+//   conversions and roundings   1e-6 of every term, margins 1e-5 of every term;
+//   flushed or subnormal k, m   2^-124, against p > 2^-63 / gamma (c2 > 2^-60, r > 1/4),
+//                               whose margin is 1e-5 p, and c > 2^-30;
+//   subnormal inv_dx            2^-150 times |u| < 500 c (p > slack), against
+//                               sidx > 2^-110;
+//   subnormal advection term    2^-149, against c sidx > 2^-100.
+// Overflows give infinities or NaN, and those the answer false.
 template <int ND>
 __device__ __forceinline__ bool speed_below(const double (&u)[ND + 2], double rb, double pb, float gam,
                                             const float (&inv_dx)[3], float below)
 {
-    const float r0 = cut_f32(u[0]), rbf = cut_f32(rb), pbf = cut_f32(pb), e = cut_f32(u[ND + 1]);
+    const int ref = __double2hiint(__double_as_longlong(rb) != 0 ? rb : u[0]) & 0x7ff00000;
+    const int bias = min(max(ref - 0x07f00000, 0x00100000), 0x70000000);
+    const float r0 = cut_f32(u[0], bias), rbf = cut_f32(rb, bias), pbf = cut_f32(pb, bias), e = cut_f32(u[ND + 1], bias);
     const float r = rbf + r0;
     const float rinv = __fdividef(1.0f, r);
     float m2 = 0.0f, adv = 0.0f, sidx = 0.0f;
 #pragma unroll
     for (int d = 0; d < ND; ++d) {
-        const float m = fabsf(cut_f32(u[1 + d]));
+        const float m = fabsf(cut_f32(u[1 + d], bias));
         m2 = fmaf(m, m, m2);
         adv = fmaf(m, inv_dx[d], adv);
         sidx += inv_dx[d];
@@ -304,8 +319,10 @@ __device__ __forceinline__ bool speed_below(const double (&u)[ND + 2], double rb
     const float p = pbf + (gam - 1.0f) * (e - k);
     const float slack = 1e-5f * (fabsf(pbf) + gam * (fabsf(e) + k));
     const float c2 = gam * (p + slack) * rinv;
-    const float s = 1.00001f * fmaf(adv, rinv, c2 * rsqrtf(c2) * sidx);
-    return r > 0.25f * (fabsf(rbf) + fabsf(r0)) && r < 1e30f && p > slack && s < below;
+    const float csidx = c2 * rsqrtf(c2) * sidx;
+    const float s = 1.00001f * fmaf(adv, rinv, csidx);
+    return r > 0.25f * (fabsf(rbf) + fabsf(r0)) && r > 0.25f && r < 1e30f && p > slack && c2 > 0x1p-60f
+        && csidx > 0x1p-100f && sidx > 0x1p-110f && s < below;
 }
 
 // Background seen by one cell in HSE mode (all zero in plain mode).
