@@ -759,14 +759,18 @@ __device__ __forceinline__ double block_max_t(T v, double *red)
     return double(v);
 }
 
-// First act of a step kernel (launch_step): waits for the kernel before
-// it in the stream to end, its writes visible, then lets the next one's CTAs
-// take SMs as this kernel's leave them.  Nothing of the previous step is read
-// before the wait.  Without a chained launch both are no-ops.
+// First act of a step kernel (launch_step): waits for the kernel before it in
+// the stream to end, its writes visible.  Nothing of the previous step is read
+// before the wait; without a chained launch it is a no-op.  The next kernel's
+// CTAs are let in as this one's exit, not by an earlier
+// griddepcontrol.launch_dependents: placed while this kernel's CTAs still
+// hold their slots, they pile up on the slots a grid of less than full
+// residency leaves open, and the SMs then get unequal shares (FP32, us per
+// step, early -> at exit: 288 CTAs of 96^3 on 456 slots 75.3 -> 58.2, 256 of 64^3
+// 33.9 -> 27.7, 2D 384^2 12.2 -> 10.7; full grids gain 0 to 2 %).
 __device__ __forceinline__ void chain_begin()
 {
     asm volatile("griddepcontrol.wait;" ::: "memory");
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 
 // Last-CTA finalisation of a step's time control.  Each of the nblocks

@@ -113,11 +113,11 @@ cudaError_t persistent_grid(PerDeviceInt &cache, K kernel, size_t smem, int thre
     }, max_grid);
 }
 
-// Launches a step kernel.  CHAIN: its CTAs may be placed while the kernel before
-// it in the stream drains (programmatic dependent launch; the kernel waits in
+// Launches a step kernel.  CHAIN: it may begin as the CTAs of the kernel before
+// it in the stream exit (programmatic dependent launch; the kernel waits in
 // chain_begin), so that steps follow one another without the gap of a launch: us
-// per step, plain -> chained, FP32 32^3 15.8 -> 13.9, 2D FP64 128^2 24.6 -> 23.1,
-// 2D FP32 2048^2 104.0 -> 101.7.  The FP64 3D steps (200 us and more, one CTA per
+// per step, plain -> chained, FP32 32^3 15.9 -> 13.6, 2D FP64 128^2 24.6 -> 22.9,
+// 2D FP32 2048^2 104.1 -> 101.6.  The FP64 3D steps (200 us and more, one CTA per
 // SM) gain nothing and are launched plainly.
 template <bool CHAIN, typename K, typename A>
 cudaError_t launch_step(K kernel, dim3 grid, int threads, size_t smem, cudaStream_t stream, const A &args)
