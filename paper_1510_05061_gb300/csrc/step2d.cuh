@@ -317,9 +317,12 @@ __device__ __forceinline__ void step2d_body(const StepArgs &a, int tile, double 
 
 // FP64: 24 resident warps per SM (80 registers) keep the FP64 pipe fed while
 // other warps run the slopes' and roots' integer work (517x331: 110.9 us with
-// 16 warps, 90 registers).
+// 16 warps, 90 registers).  FP32: no request (0), with which the compiler takes
+// 32 to 40 registers, 48 and more warps; asked for one CTA it takes 55, and grids
+// of several waves, bound by instruction issue, lose (40 x 30000: 80.0 us against
+// 65.2, 256 x 4000 45.6 against 37.1).
 template <typename T, int TX, int TY, int ST = STAGE_HANCOCK, int RC = RECON_PLM>
-__global__ void __launch_bounds__(TX * TY, sizeof(T) == 8 ? 768 / (TX * TY) : 1) step2d_kernel(const StepArgs a)
+__global__ void __launch_bounds__(TX * TY, sizeof(T) == 8 ? 768 / (TX * TY) : 0) step2d_kernel(const StepArgs a)
 {
     constexpr int NT = TX * TY;
     extern __shared__ __align__(16) unsigned char smem_raw[];
