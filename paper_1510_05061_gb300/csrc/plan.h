@@ -99,10 +99,13 @@ struct Plan2D {
 // against 160 with 32 x 8; 517x331 111 against 117), 16 x 8 while those fit one
 // per SM (128^2: 26 against 33); FP32 32 x 16 (384^2 12.6 against 14.5), 16 x 16
 // for the parabolic stages (1448^2 179 against 187).  A strip (linear states)
-// is taken where its modelled time, row time x (rows per CTA + 2.2), is below
-// the tiles' time per padded cell; the row times at full residency and the
-// tiles' cell times are fitted at 512^2 to 2048^2.  The crossing lies near 700^2
-// (FP64: 266 against 293) and 1024^2 (FP32: 38.3 against 37.9).
+// is taken where its modelled time, base + row x rows per CTA, is below the
+// tiles', a constant and a time per padded cell.  FP64: fitted at 512^2 to 2048^2;
+// the crossing lies near 700^2 (266 against 293).  FP32: fitted to 46 shapes from
+// 61^2 to 2048^2, 40 x 30000 and 2600 x 48 within 6 %, the tiles' time taken 3 %
+// short so that the Runge-Kutta stages, whose strips cost a little more, gain too;
+// us, strip and tile: 600^2 19.7 and 18.3, 2600 x 100 18.6 and 15.9, 800 x 700 25.5
+// and 23.7, 250 x 2600 24.6 and 27.6, 1024^2 36.1 and 37.4, 2048^2 101 and 129.
 inline Plan2D plan2d(int nx, int ny, bool fp32, bool ppm)
 {
     constexpr int SMS = 152;
@@ -111,13 +114,13 @@ inline Plan2D plan2d(int nx, int ny, bool fp32, bool ppm)
     if (!fp32 && along(nx, 16) * along(ny, 8) <= SMS) best.ty = 8;
     if (ppm) return best;
     const double cells = (double)along(nx, best.tx) * best.tx * along(ny, best.ty) * best.ty;
-    double tbest = fp32 ? 4.0 + 31.5e-6 * cells : 10.0 + 525e-6 * cells;
-    struct Strip { int nt, ctas; double row; };
-    static const Strip f64[] = {{128, 3, 22.9}};
-    static const Strip f32[] = {{128, 6, 2.5}, {256, 3, 2.5}};
+    double tbest = fp32 ? 7.8 + 28.9e-6 * cells : 10.0 + 525e-6 * cells;
+    struct Strip { int nt, ctas; double base, row; };
+    static const Strip f64[] = {{128, 3, 50.4, 22.9}};
+    static const Strip f32[] = {{128, 6, 13.0, 2.1}, {256, 3, 11.5, 2.15}};
     const Strip *c = fp32 ? f32 : f64;
     for (int i = 0; i < (fp32 ? 2 : 1); ++i) {
-        const double t = c[i].row * (along(along(nx, c[i].nt - 4) * ny, SMS * c[i].ctas) + 2.2);
+        const double t = c[i].base + c[i].row * along(along(nx, c[i].nt - 4) * ny, SMS * c[i].ctas);
         if (t < tbest) {
             tbest = t;
             best.march = c[i].nt;
