@@ -191,16 +191,9 @@ cudaError_t launch_once(hydro_batch *b, int parity)
     return e;
 }
 
-// Longest z-chunk of an instance's column: long chunks re-read few halo
-// planes (4 per chunk), and the largest-first claim order keeps the SMs
-// balanced even when whole columns are single items.
-constexpr int BATCH_ZCHUNK_DEFAULT = 64;
-
 int zchunk_of(const hydro_batch *b, const hydro_problem &p)
 {
-    const int zmax = b->zchunk > 0 ? b->zchunk : BATCH_ZCHUNK_DEFAULT;
-    const int nch = (p.n[2] + zmax - 1) / zmax;       // chunks of (nearly) equal length
-    return (p.n[2] + nch - 1) / nch;
+    return batch_chunk(p.n[2], b->zchunk > 0 ? b->zchunk : BATCH_ZCHUNK_DEFAULT);
 }
 
 // Staging buffer k ready for rewriting and holding at least `need` bytes.
@@ -235,7 +228,9 @@ int rebuild(hydro_batch *b)
         std::vector<const hydro_problem *> p3;
         for (const InstInfo &I : b->inst)
             if (I.active && I.prob.ndim == 3) p3.push_back(&I.prob);
-        if (!p3.empty()) plan = batch_plan(p3.data(), (int)p3.size(), b->precision == HYDRO_FP32, b->pick ? -1 : b->variant);
+        const bool fp32 = b->precision == HYDRO_FP32;
+        if (!p3.empty()) plan = batch_plan(p3.data(), (int)p3.size(), fp32, b->pick ? -1 : b->variant);
+        if (fp32 && plan.shares > 0 && !shares_pay(plan, p3.data(), (int)p3.size(), b->variant)) plan.shares = 0;
         if (plan.shares > 0) b->variant = plan.variant;
     }
     const TileShape ts = TILE3D_SHAPES[b->variant];

@@ -36,18 +36,19 @@ struct BatchPlan {
 // march neighbouring tiles at the same heights and find each other's halo rows
 // in L2 (default_plan's line; 126 MB: 362 shared, 394 in chunks; 344 MB 1310 and
 // 1136; 1.3 GB 4200 and 3641).
+constexpr TileCost BATCH_F64[3] = {{2, 1, 24.0, 24.0, 2.0}, {0, 1, 28.2, 28.2, 2.0}, {1, 1, 19.5, 19.5, 2.0}};
+constexpr TileCost BATCH_F32[3] = {{2, 2, 3.5, 1.8, 3.0}, {7, 1, 3.5, 3.5, 3.0}, {1, 2, 2.5, 1.0, 3.0}};
+
 inline BatchPlan batch_plan(const hydro_problem *const *p, int count, bool fp32, int only)
 {
     constexpr int SMS = 152;
-    static const TileCost f64[] = {{2, 1, 24.0, 24.0, 2.0}, {0, 1, 28.2, 28.2, 2.0}, {1, 1, 19.5, 19.5, 2.0}};
-    static const TileCost f32[] = {{2, 2, 3.5, 1.8, 3.0}, {7, 1, 3.5, 3.5, 3.0}, {1, 2, 2.5, 1.0, 3.0}};
     BatchPlan best{};
     double tbest = 0.0, cells = 0.0;
     for (int j = 0; j < count; ++j) cells += (double)p[j]->n[0] * p[j]->n[1] * p[j]->n[2];
     if (fp32 && cells * 5 * 4 > 160e6) return best;
     const bool beyond_l2 = fp32 && 2 * cells * 5 * 4 > 129e6;
     for (int i = 0; i < 3; ++i) {
-        const TileCost &c = fp32 ? f32[i] : f64[i];
+        const TileCost &c = fp32 ? BATCH_F32[i] : BATCH_F64[i];
         if (only >= 0 ? only % 4 != c.variant % 4 : beyond_l2 && i != 1) continue;
         const TileShape s = TILE3D_SHAPES[c.variant];
         long long cols = 0, W = 0;
@@ -66,6 +67,53 @@ inline BatchPlan batch_plan(const hydro_problem *const *p, int count, bool fp32,
         }
     }
     return best;
+}
+
+// Longest z-chunk of an instance's column where the columns are claimed in
+// chunks of nearly equal length: long chunks re-read few halo planes (4 per
+// chunk), and the largest-first claim order keeps the SMs balanced even when
+// whole columns are single items.
+constexpr int BATCH_ZCHUNK_DEFAULT = 64;
+
+inline int batch_chunk(int nz, int longest)
+{
+    const int nch = (nz + longest - 1) / longest;
+    return (nz + nch - 1) / nch;
+}
+
+// Whether an FP32 batch takes the plan's shares rather than chunks with the
+// tile of variant `otherwise`.  The shares cut the columns into more pieces,
+// each costing `fixed` planes: a batch that has the chip to itself gains (the
+// CTAs end together), but where several batches step on streams of their own,
+// idle CTAs are filled by the others and only the work counts.  So the shares
+// are taken where their modelled work is no more than the chunks', or where the
+// chunks are too few to fill half of the CTAs.  Three batches at once, shares
+// against chunks, at a ratio of modelled works of 0.956 (5 boxes of 35^3 to
+// 115^3): 0.952, 0.969 (24^3 to 123^3): 0.937, 1.008: 1.010, 1.03: 1.03; half
+// filled 1.02 to 3.2.  Alone the shares' gain is 1.1 to 1.4 where they are given
+// up, 1.07 to 4.9 where they stay.  The 16 x 16 tile's halo rows cost 3 % more
+// where three batches' buffers are well beyond the L2 (from 100 MB each).
+inline bool shares_pay(const BatchPlan &plan, const hydro_problem *const *p, int count, int otherwise)
+{
+    constexpr int SMS = 152;
+    const TileCost *s = nullptr, *c = nullptr;
+    for (const TileCost &t : BATCH_F32) {
+        if (t.variant % 4 == plan.variant % 4) s = &t;
+        if (t.variant % 4 == otherwise % 4) c = &t;
+    }
+    if (!s || !c) return s != nullptr;
+    const TileShape ss = TILE3D_SHAPES[plan.variant], cs = TILE3D_SHAPES[otherwise];
+    double bytes = 0.0, shares = plan.fixed * plan.shares, chunks = 0.0, longest = 0.0;
+    for (int j = 0; j < count; ++j) {
+        const int *n = p[j]->n, zc = batch_chunk(n[2], BATCH_ZCHUNK_DEFAULT);
+        const auto tiles = [n](const TileShape &t) { return (double)((n[0] + t.tx - 1) / t.tx) * ((n[1] + t.ty - 1) / t.ty); };
+        bytes += 2.0 * 5 * 4 * n[0] * n[1] * n[2];
+        shares += tiles(ss) * (n[2] + plan.fixed);
+        chunks += tiles(cs) * (n[2] + c->fixed * ((n[2] + zc - 1) / zc));
+        longest = std::max(longest, zc + c->fixed);
+    }
+    const double spill = plan.variant % 4 == 2 && bytes > 100e6 ? 1.03 : 1.0;
+    return 0.99 * spill * s->unit * shares <= c->unit * chunks || chunks < 0.5 * SMS * c->ctas * longest;
 }
 
 // The 3D columns of a batch cut into equal shares (batch_plan), one for each
