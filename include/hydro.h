@@ -183,8 +183,10 @@ int hydro_get_fields(hydro_sim *sim, int what, double *host_dst);
    from the host. */
 int hydro_debug_poke(hydro_sim *sim, int var, long cell, double v);
 
-/* Select the 3D z-chunk length (planes per CTA); 0 restores the default
-   (the balanced grid; z-chunks for the paired-cell variants).
+/* Select the 3D z-chunk length (planes per CTA); 0 restores the default of the
+   selected tile, chosen from the grid's size: z-chunks of one piece per CTA, the
+   balanced grid, or (always for the paired-cell variants) z-chunks in several
+   waves.  Until a length is selected, hydro_set_tile takes the new tile's default.
    A negative value selects the balanced grid instead: as many CTAs as the
    device holds resident at once, the (tile, z-chunk) pieces taken in whole
    waves of neighbouring tiles at the same heights while at least one wave

@@ -46,6 +46,7 @@ struct hydro_sim {
     int variant;             // 3D tile shape (TILE3D_SHAPES index)
     int zchunk;
     int balanced;            // 3D: 0, or the balanced grid's z-chunk setting (-1: whole columns, -Z)
+    bool default_z;          // 3D: the z partition is the default one (a new tile takes its own)
     long launches;
     int err_state;           // sticky host-side copy of a non-physical error
     std::vector<PlaneBG> bg_host;
@@ -207,7 +208,8 @@ AuxArgs aux_args(const hydro_sim *s, void *U)
     return a;
 }
 
-// z-chunk of the kernels without a balanced grid (the paired-cell tiles)
+// z-chunks in several waves: the paired-cell tiles, which have no balanced
+// grid, and the tiles tile_zchunk leaves them to
 int default_zchunk(const hydro_sim *s)
 {
     if (s->prob.ndim == 2) return 1;
@@ -221,13 +223,16 @@ int default_zchunk(const hydro_sim *s)
     return (int)((nz + nch - 1) / nch);
 }
 
-// The default z partition: the plan's, where the kernel has it.
+// The default z partition of the solve's tile: the plan's for its own tile,
+// one made for the tile the caller chose otherwise.
 void set_default_partition(hydro_sim *s)
 {
+    s->default_z = true;
     s->balanced = 0;
     s->zchunk = default_zchunk(s);
     if (s->prob.scheme == HYDRO_SCHEME_CTU || pair_variant(s->variant)) return;
-    const int z = default_plan(s->prob).zchunk;
+    const LaunchPlan plan = default_plan(s->prob);
+    const int z = s->variant == plan.variant ? plan.zchunk : tile_zchunk(s->prob, s->variant);
     if (z > 0) s->zchunk = z;
     else s->balanced = z;
 }
@@ -643,6 +648,7 @@ int hydro_set_zchunk(hydro_sim *s, int zchunk)
         if (s->prob.ndim != 3 || s->prob.scheme == HYDRO_SCHEME_CTU || pair_variant(s->variant))
             return HYDRO_ERR_INVALID_ARG;
         s->balanced = std::max(zchunk, -s->prob.n[2]);   // chunks of at most nz planes
+        s->default_z = false;
         return HYDRO_OK;
     }
     if (s->prob.ndim == 2) return zchunk <= 1 ? HYDRO_OK : HYDRO_ERR_INVALID_ARG;
@@ -652,6 +658,7 @@ int hydro_set_zchunk(hydro_sim *s, int zchunk)
     }
     s->zchunk = std::min(zchunk, s->prob.n[2]);
     s->balanced = 0;
+    s->default_z = false;
     return HYDRO_OK;
 }
 
@@ -672,6 +679,7 @@ int hydro_set_tile(hydro_sim *s, int variant)
     if (pair_variant(variant)) s->balanced = 0;   // the paired kernel has z-chunks only
     s->tiles_x = tiles_along(s->prob.n[0], tile_shape(variant).tx);
     s->tiles_y = tiles_along(s->prob.n[1], tile_shape(variant).ty);
+    if (s->default_z) set_default_partition(s);
     return HYDRO_OK;
 }
 

@@ -89,6 +89,36 @@ inline LaunchPlan default_plan(const hydro_problem &p)
     return best;
 }
 
+// z partition of the tile of variant v chosen by the caller: planes per CTA,
+// -1 for the balanced grid, or 0 for chunks in several waves (the caller's).
+// One piece per CTA where a single wave of the kernel's resident CTAs holds every
+// tile and the balanced grid would split columns, else the balanced grid, as in
+// default_plan.  Measured on 24^3 to 320^3, us, several-wave chunks -> this:
+// FP32 24^3 25 to 38 -> 13 to 16, 96^3 56 to 79 -> 54 to 66, 128^3 122 to 179 -> 112 to
+// 142, FP64 64^3 234 to 344 -> 234 to 324.  The FP32 32 x 8 tile keeps those chunks
+// where the state's buffers pass 110 MB, the 16 x 16 tile where they pass 250 MB:
+// their neighbouring tiles march at the same heights and find each other's halo
+// rows in L2 (32 x 8, 192^3: 337 against 355, Runge-Kutta 660 against 864).
+inline int tile_zchunk(const hydro_problem &p, int v)
+{
+    constexpr int SMS = 152;
+    const TileShape s = TILE3D_SHAPES[v];
+    const bool fp32 = p.precision == HYDRO_FP32, rk = p.scheme != HYDRO_SCHEME_HANCOCK, ppm = p.recon == HYDRO_RECON_PPM;
+    const bool async = v >= 4 && !rk;
+    const int shape = v % 4;
+    // resident CTAs that share an SM without loss
+    const int k = !fp32 || shape == 3 ? 1 : (shape == 0 && !async && !ppm ? 3 : (shape == 2 && ppm ? 1 : 2));
+    const double buffers = (rk ? 3.0 : 2.0) * 5 * (fp32 ? 4 : 8) * p.n[0] * p.n[1] * p.n[2];
+    if (fp32 && !async && !ppm && ((shape == 0 && buffers > 110e6) || (shape == 2 && buffers > 250e6))) return 0;
+    const long long T = (long long)((p.n[0] + s.tx - 1) / s.tx) * ((p.n[1] + s.ty - 1) / s.ty), G = (long long)SMS * k;
+    const long long planes = (T * p.n[2] + G - 1) / G;
+    if (T > G) return -1;
+    const double fixed = ppm ? 1.8 : 1.2;
+    const bool split = planes > 1 && !(G % T == 0 && p.n[2] % (G / T) == 0);
+    const int zc = (int)((p.n[2] + G / T - 1) / (G / T));
+    return zc + fixed < planes + (split ? 2 : 1) * fixed ? zc : -1;
+}
+
 // Launch shape of the 2D step: march = threads of a marched strip, or 0 and
 // the tile (tx x ty).
 struct Plan2D {
