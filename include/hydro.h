@@ -347,11 +347,12 @@ int hydro_batch_init(const hydro_problem *probs, int count, void *const *Ua, voi
 
 /* Select the 3D tile shape and staging depth (variant index, see
    hydro_set_tile; variants 3 and 7 are FP32 only) and the longest z-chunk
-   of an instance's column (0 = default, 64 planes; each column is cut into
-   chunks of nearly equal length).  Until it is called, a batch made by
-   hydro_batch_init takes a tile fitted to its sizes and shares the columns out
-   evenly, and one made by hydro_batch_create variant 7 (FP64: 6) and chunks of
-   64 planes.  Rebuilds the work lists (and the graph
+   of an instance's column (each column is cut into chunks of nearly equal
+   length).  0 is the default: chunks of at most 64 planes, or, in a batch made by
+   hydro_batch_init, the columns shared out evenly where that pays.  Until it is
+   called, a batch made by hydro_batch_init takes a tile fitted to its sizes, and
+   one made by hydro_batch_create variant 7 (FP64: 6), both with z-chunk 0.
+   Rebuilds the work lists (and the graph
    when the kernel changes).  Results do not depend on this choice.
    hydro_batch_variant_shape gives a variant's tile shape (tx x ty);
    variants v and v + 4 share it. */

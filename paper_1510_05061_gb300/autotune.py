@@ -20,8 +20,14 @@ from typing import Dict, Iterable, Optional
 
 from . import inputs
 
-# longest z-chunk of an instance's column in a batch (shorter columns are one item)
-DEFAULT_ZCHUNKS = (16, 32, 64, 128, 256)
+# longest z-chunk of an instance's column in a batch (shorter columns are one
+# item); 0: the tile's default partition
+DEFAULT_ZCHUNKS = (0, 16, 32, 64, 128, 256)
+
+
+def distinct_variants(variants, precision) -> list:
+    """FP64 kernels stage alike in variants v and v + 4: one of each is timed."""
+    return [v for v in variants if precision == inputs.FP32 or v < 4]
 
 
 def cache_path() -> str:
@@ -111,7 +117,7 @@ def tune_batch(batch, steps: int = 4, zchunks: Iterable[int] = DEFAULT_ZCHUNKS,
         batch.configure(ch["variant"], ch["zchunk"])
         return dict(ch, cached=True)
     shapes = hydro.batch_variants()
-    variants = list(range(len(shapes))) if variants is None else list(variants)
+    variants = distinct_variants(range(len(shapes)), batch.probs[0].precision) if variants is None else list(variants)
     table = []
     best = None
     for v in variants:
@@ -161,11 +167,11 @@ def time_sim_steps(sim, steps: int) -> float:
     return a.elapsed_time(b) / steps
 
 
-def tune_simulation(sim, steps: int = 3, zchunks: Iterable[int] = (16, 32, 64, 128, -1, -64, -128),
+def tune_simulation(sim, steps: int = 3, zchunks: Iterable[int] = (0, 16, 32, 64, 128, -1, -64, -128),
                     variants: Optional[Iterable[int]] = None, use_cache: bool = True) -> dict:
     """Configure a single 3D solve with its fastest (tile shape, z-chunk);
-    a negative z-chunk is the balanced grid (-1, hydro.ZCHUNK_BALANCED: over
-    whole columns; -Z: over Z-plane chunks).  Tuning advances the solve by the
+    z-chunk 0 is the tile's default partition, a negative one the balanced grid
+    (-1, hydro.ZCHUNK_BALANCED: over whole columns; -Z: over Z-plane chunks).  Tuning advances the solve by the
     steps it times."""
     from . import hydro
 
@@ -179,7 +185,7 @@ def tune_simulation(sim, steps: int = 3, zchunks: Iterable[int] = (16, 32, 64, 1
         sim.configure(ch["variant"], ch["zchunk"])
         return dict(ch, cached=True)
     shapes = dict(hydro.sim_variants())
-    variants = sorted(shapes) if variants is None else list(variants)
+    variants = distinct_variants(sorted(shapes), sim.prob.precision) if variants is None else list(variants)
     table, best = [], None
     for v in variants:
         for z in zchunks:

@@ -147,6 +147,7 @@ struct hydro_batch {
     cudaStream_t stream;
     int parity;                // parity of the next launch
     int variant, zchunk;       // zchunk: longest chunk of an instance's column (0 = default)
+    bool fixed;                // made by hydro_batch_init: the default is batch_plan's, not chunks
     bool even, pick;           // columns in equal shares (batch_plan), and the variant of its choice
     bool dirty;                // queue / tables need an upload
     bool use_graph;
@@ -672,7 +673,7 @@ int hydro_batch_init(const hydro_problem *probs, int count, void *const *Ua, voi
         if (rc) break;
         w += inst_layout(probs[i]).total;
     }
-    b->even = b->pick = true;
+    b->fixed = b->even = b->pick = true;
     if (rc == HYDRO_OK) rc = rebuild(b);
     b->pick = false;   // later changes of membership keep the kernel
     if (rc) {
@@ -688,7 +689,7 @@ int hydro_batch_configure(hydro_batch *b, int variant, int zchunk)
     if (!b || !tile3d_available(variant, b->precision == HYDRO_FP32) || zchunk < 0) return HYDRO_ERR_INVALID_ARG;
     b->variant = variant;
     b->zchunk = zchunk;
-    b->even = false;
+    b->even = b->fixed && zchunk == 0;
     return rebuild(b);
 }
 
