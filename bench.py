@@ -65,7 +65,7 @@ FLOPS_PER_ZONE_2D_PPM = 2 * 372 + 8 + 19
 FLOPS_PER_ZONE_3D_CTU = 13 + 75 + 3 * 35 + 60 + 216 + 3 * 2 * 42 + 216 + 70 + 25
 FLOPS_PER_ZONE_2D_CTU = 10 + 40 + 2 * 25 + 32 + 128 + 2 * 2 * 26 + 128 + 42 + 19
 
-# tile shape of each 3D variant; variants 4..7 stage the next plane asynchronously
+# tile shape of each 3D variant; FP32 variants 4..7 stage the next plane asynchronously
 TILE_NAMES = {0: "32, 8", 1: "32, 4", 2: "16, 16", 3: "32, 16", 4: "32, 8", 5: "32, 4", 6: "16, 16", 7: "32, 16"}
 # paired-cell FP32 variants: threads (x, y) per tile (two x-adjacent cells per thread)
 PAIR_THREADS = {8: (16, 16), 9: (16, 8), 10: (8, 16)}
@@ -126,9 +126,10 @@ def step_kernel_names(prob, variant: int):
     tname = "double" if itemsize == 8 else "float"
     stages = (1, 2) if rk2 else (0,)
     # template arguments: stage, reconstruction, staging depth (the tuned one
-    # for the MUSCL-Hancock step, the precision's default for the stages),
-    # and whether the FP64 MUSCL-Hancock step takes the kernel for gravity
-    # along z only (without the x and y gravity terms)
+    # for the MUSCL-Hancock step, the precision's default for the stages; an
+    # FP64 solve launches variants 0..3 only, launched_kernels), and whether the
+    # FP64 MUSCL-Hancock step takes the kernel for gravity along z only (without
+    # the x and y gravity terms)
     async_flag = int(variant >= 4) if not rk2 else int(itemsize == 8)
     gz = int(itemsize == 8 and not rk2 and bool(prob.hse_subtract or (prob.grav[0] == 0 and prob.grav[1] == 0)))
     if prob.scheme == inputs.CTU:
@@ -141,7 +142,28 @@ def step_kernel_names(prob, variant: int):
         minb = 2 if variant == 8 else 3
         return [f"step3d_pair_kernel<{prob.hse_subtract}, {txp}, {typ}, {pgz}, {minb}>"]
     return [(f"step3d_kernel<{tname}, {prob.hse_subtract}, {tile}, {st}, {prob.recon}, {async_flag}, {gz}>"
-             if prob.ndim == 3 else f"step2d_kernel<{tname}, 32, 8, {st}, {prob.recon}>") for st in stages]
+             if prob.ndim == 3 else f"step2d_kernel<{tname}, stage {st}> or march2d_kernel (by size)") for st in stages]
+
+
+def launched_kernels(prob, variant: int):
+    """step_kernel_names of the kernels `variant` launches: an FP64 solve has one
+    kernel for variants v and v + 4, and the corner transport upwind step's
+    last argument says whether the x and y gravity terms are left out."""
+    if prob.precision == inputs.FP64:
+        variant %= 4
+    names = step_kernel_names(prob, variant)
+    if prob.scheme == inputs.CTU and prob.ndim == 3:
+        gz = int(prob.precision == inputs.FP64 and bool(prob.hse_subtract or (prob.grav[0] == 0 and prob.grav[1] == 0)))
+        names = [f"{n[:-1]}, {gz}>" for n in names]
+    return names
+
+
+def traffic_key(kernel: str) -> str:
+    """The key of a kernel in profiles/traffic.json: its name as step_kernel_names
+    has it (the corner transport upwind step without its last argument)."""
+    if kernel.startswith("ctu3d_kernel<") and kernel.count(",") == 4:
+        return kernel[:kernel.rindex(",")] + ">"
+    return kernel
 
 
 # translation units that compile (and launch) each kernel family; a kernel's
@@ -152,6 +174,7 @@ KERNEL_UNITS = {
     "step3d_batch_kernel": ("batch3d_f64.cu", "batch3d_f32.cu"),
     "step2d_kernel": ("step2d.cu",),
     "step2d_batch_kernel": ("batch2d.cu",),
+    "march2d_kernel": ("march2d.cu",),
     "ctu3d_kernel": ("ctu3d.cu",),
     "ctu2d_kernel": ("ctu2d.cu",),
 }
@@ -203,7 +226,7 @@ def measured_traffic(config: str, kernel: str):
             table = json.load(fh)
     except (OSError, ValueError):
         return None
-    e = table.get(config, {}).get(kernel)
+    e = table.get(config, {}).get(traffic_key(kernel))
     if not e or e.get("source_sha") != kernel_source_sha(kernel):
         return None
     return float(e["bytes_per_launch"])
@@ -250,7 +273,7 @@ def record_traffic(config: str, csv_path: str, scale: float = 1.0, note: str = "
                  "source_sha": kernel_source_sha(name)}
         if scale != 1.0:
             entry["scaled"] = note or f"captured on a smaller grid, bytes x {scale:g}"
-        table.setdefault(config, {})[name] = entry
+        table.setdefault(config, {})[traffic_key(name)] = entry
     with open(path, "w") as fh:
         json.dump(table, fh, indent=1, sort_keys=True)
     print("| kernel | launches | device time (ms) | share | DRAM bytes per launch |")
@@ -750,7 +773,7 @@ def run_gpu_slabs(args):
         sim.configure(tune["variant"], tune["zchunk"])
     slabs = hydro.Slabs(prob, W, R, stream=stream)
     if tune is not None:
-        slabs.configure(tune["variant"], tune["zchunk"])
+        slabs.configure(tune["variant"], tune["zchunk"] or hydro.ZCHUNK_BALANCED)   # (slabs have no fitted default)
 
     def timed(step):
         for _ in range(args.warmup):
@@ -917,8 +940,8 @@ def run_gpu(args):
     achieved_gbs = bytes_per_zone * zones_per_launch / (kern_avg_ms * 1e-3) / 1e9
     hbm_peak = float(peaks.get("hbm_gbs", 6800.0))
     clocks = clk.summary()
-    variant = tune["variant"] if tune else (0 if itemsize == 4 else 4)
-    knames = step_kernel_names(prob, variant)
+    variant = tune["variant"] if tune else (0 if itemsize == 4 else 2)
+    knames = launched_kernels(prob, variant)
     kname = " + ".join(knames)
     # DRAM bytes of one step: the sum over its kernels (null if any is missing or stale)
     traffic = args.traffic
