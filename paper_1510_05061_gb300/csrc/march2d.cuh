@@ -15,7 +15,7 @@
 // 4 of NT columns and two predicted rows per piece, so it pays on large grids
 // (plan2d in plan.h).  What bounds it is what bounds the tiles: the FP64 pipe,
 // or instruction issue in FP32.  Measured on GB300, us per MUSCL-Hancock step:
-// FP32 2048^2 137.5 (32 x 8 tile) -> 103, 1448^2 68.4 (32 x 16 tile) -> 55.5;
+// FP32 2048^2 128.7 (32 x 16 tile) -> 101, 1448^2 67.4 -> 53.3;
 // FP64 1448^2 1114 (16 x 16 tile) -> 965.  Linear states only: the parabolic
 // stages' five rows in registers cost what the march saves (FP32 1448^2 179 us
 // a step for both, FP64 724^2 1048 against 1072).

@@ -74,6 +74,8 @@ constexpr int STEP3D_HELPERS = sizeof(T) == 8 ? 128 : 0;
 template <typename T, int TX, int TY>
 constexpr int STEP3D_THREADS = TX * TY + STEP3D_HELPERS<T>;
 
+// AS: asynchronous staging (FP32; the FP64 kernels' helper warps stage either
+// way, the argument only names their stage kernels).
 template <typename T, bool HSE, int TX, int TY, int RC = RECON_PLM, bool AS = (sizeof(T) == 8)>
 struct Step3DSmem {
     static constexpr int NV = 5;
@@ -123,12 +125,12 @@ struct Step3DSmem {
     static constexpr size_t rest = 2 * wx + 2 * wy + fx + fy + dif + raw;
     // (fits: one CTA's limit, and the tile's resident CTAs per SM, each with
     // about 1.5 KB of reserved and static shared memory, in the SM's 228 KB).
-    // Measured on GB300: +4..+21 % for the synchronous FP32 tiles and +4 %
-    // for FP64 PPM; -5 % for the FP32 32 x 16 tile with asynchronous staging
-    // and -0.4 % for the FP64 PLM tiles, which keep the plain ring.
+    // Measured on GB300: +4..+21 % for the synchronous FP32 tiles, -5 % for the
+    // FP32 32 x 16 tile with asynchronous staging, which keeps the plain ring.
+    // The FP64 helper warps stage into the spare slot and need it.
     static constexpr size_t spare_bytes = ((NRS + 1) * plane + rest) * sizeof(T);
     static constexpr bool spare = spare_bytes <= 226 * 1024 && ctas * (spare_bytes + 1536) <= 228 * 1024
-                               && (!async || (sizeof(T) == 8 && RC == RECON_PPM));
+                               && !async;
     static constexpr int NR = NRS + (spare ? 1 : 0);
     static constexpr size_t prim = (size_t)NR * plane;          // [NR][NV][HY][HXS]
     static constexpr size_t elems = prim + rest;
@@ -887,7 +889,7 @@ __device__ __forceinline__ void step3d_body(const StepArgs &a, int tile, int z0,
             // them packed on the first TX + TY threads, which measured faster
             // there (the other form compiled to fewer registers and less ILP).
             constexpr bool split = NT <= 256;
-            if (!WS && (split ? (tid < TY || (tid >= 32 && tid < 32 + TX)) : tid < TY + TX)) {
+            if (split ? (tid < TY || (tid >= 32 && tid < 32 + TX)) : tid < TY + TX) {
                 const bool isx = tid < TY;
                 const int r = isx ? tid : (split ? tid - 32 : tid - TY);
                 T wl[NV], wr[NV], f[NV];
