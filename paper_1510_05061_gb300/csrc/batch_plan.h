@@ -86,13 +86,17 @@ inline int batch_chunk(int nz, int longest)
 // each costing `fixed` planes: a batch that has the chip to itself gains (the
 // CTAs end together), but where several batches step on streams of their own,
 // idle CTAs are filled by the others and only the work counts.  So the shares
-// are taken where their modelled work is no more than the chunks', or where the
-// chunks are too few to fill half of the CTAs.  Three batches at once, shares
+// are taken where their modelled work is no more than the chunks', or where even
+// three batches' chunks leave CTAs idle (busy, the part of one batch's CTAs that
+// its chunks keep working, below a third; up to a half a ratio a little below 1
+// is made up: at 0.42 0.945: 1.010, at 0.46 0.927: 0.936).  Three batches at once, shares
 // against chunks, at a ratio of modelled works of 0.956 (5 boxes of 35^3 to
-// 115^3): 0.952, 0.969 (24^3 to 123^3): 0.937, 1.008: 1.010, 1.03: 1.03; half
-// filled 1.02 to 3.2.  Alone the shares' gain is 1.1 to 1.4 where they are given
-// up, 1.07 to 4.9 where they stay.  The 16 x 16 tile's halo rows cost 3 % more
-// where three batches' buffers are well beyond the L2 (from 100 MB each).
+// 115^3): 0.952, 0.991 (38^3 to 134^3): 0.992, 1.008: 1.010, 1.03: 1.03; busy
+// below a third 1.01 to 3.2.  Alone the shares' gain is 1.1 to 1.4 where they are given
+// up, 1.07 to 4.9 where they stay.  The 16 x 16 tile's halo rows cost 3 to 5 %
+// more where three batches' buffers are well beyond the L2 (from 100 MB each;
+// 22^3 to 112^3, ratio 1.026: 0.977); from 190 MB the shares are about 1 %
+// better than the ratio (32^3 to 128^3, 0.993: 1.004).
 inline bool shares_pay(const BatchPlan &plan, const hydro_problem *const *p, int count, int otherwise)
 {
     constexpr int SMS = 152;
@@ -112,8 +116,9 @@ inline bool shares_pay(const BatchPlan &plan, const hydro_problem *const *p, int
         chunks += tiles(cs) * (n[2] + c->fixed * ((n[2] + zc - 1) / zc));
         longest = std::max(longest, zc + c->fixed);
     }
-    const double spill = plan.variant % 4 == 2 && bytes > 100e6 ? 1.03 : 1.0;
-    return 0.99 * spill * s->unit * shares <= c->unit * chunks || chunks < 0.5 * SMS * c->ctas * longest;
+    const double spill = plan.variant % 4 == 2 && bytes > 100e6 ? 1.05 : (bytes > 190e6 ? 0.99 : 1.0);
+    const double ratio = c->unit * chunks / (spill * s->unit * shares), busy = chunks / (SMS * c->ctas * longest);
+    return busy < 1.0 / 3 || ratio >= (busy < 0.5 ? 0.92 + 0.39 * (busy - 1.0 / 3) : 1.0);
 }
 
 // The 3D columns of a batch cut into equal shares (batch_plan), one for each

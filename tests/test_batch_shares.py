@@ -33,7 +33,8 @@ int main()
 # (smallest, largest, boxes): time of three batches in turn, chunks over shares
 MEASURED = {(17, 113, 4): 2.68, (31, 67, 7): 1.31, (18, 66, 16): 1.26, (23, 99, 6): 1.09, (39, 91, 9): 1.05,
             (19, 98, 11): 1.03, (25, 96, 16): 1.02, (32, 128, 14): 1.00, (35, 115, 6): 0.952, (24, 123, 9): 0.937,
-            (36, 128, 6): 0.969, (20, 127, 10): 0.980, (39, 142, 8): 0.984, (18, 116, 14): 0.986, (27, 110, 16): 0.991}
+            (36, 128, 6): 0.969, (20, 127, 10): 0.980, (39, 142, 8): 0.984, (18, 116, 14): 0.986, (27, 110, 16): 0.991, (22, 112, 10): 0.977, (38, 134, 6): 0.992,
+            (18, 125, 5): 0.936, (18, 96, 9): 1.01, (24, 90, 5): 1.03}
 
 
 def cubes(lo, hi, n):
